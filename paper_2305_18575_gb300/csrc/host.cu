@@ -1,7 +1,7 @@
 // host.cu -- host runtime of the REI library: contexts, device memory, the
 // solve driver, result formatting, inspection calls, and the batched and
 // served forms.  Every step of the search itself runs in the kernels of
-// stage.cu and solve.cu; this file only moves inputs and results, sizes
+// stage.cu, solve.cu, relaunch.cu and slots.cu; this file only moves inputs and results, sizes
 // buffers, and launches.
 #include <cuda_runtime.h>
 
@@ -37,8 +37,8 @@ cudaError_t serve_occupancy(uint32_t threads, size_t smem, int *blocks_per_sm);
 size_t stage_smem_bytes();
 cudaError_t launch_solve(const SolveJob *job, uint32_t grid, uint32_t threads, size_t smem,
                          cudaStream_t stream);
-cudaError_t solve_occupancy(uint32_t threads, size_t smem, int *blocks_per_sm);
-cudaError_t solve_smem_max(size_t *bytes);
+cudaError_t solve_occupancy(uint32_t W, uint32_t threads, size_t smem, int *blocks_per_sm);
+cudaError_t solve_smem_max(uint32_t W, size_t *bytes);
 cudaError_t solve_batch_smem_max(size_t *bytes);
 cudaError_t launch_solve_groups(const BatchJob *jobs_dev, const GroupArgs *args, uint32_t grid, uint32_t threads,
                                 size_t smem, cudaStream_t stream);
@@ -792,7 +792,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     // launch shape
     const uint32_t seg_cap = 2 * max_cost + 4;
     size_t smem_max = 0;  // dynamic shared memory a k_solve launch can take
-    CK(solve_smem_max(&smem_max));
+    CK(solve_smem_max(W, &smem_max));
     bool gt_smem = 4ull * (n + 1 + G + max_len + 2) <= 96 * 1024;
     uint32_t warps = 16;  // (the launch bounds of k_solve)
     size_t smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps);
@@ -826,7 +826,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     }
     const uint32_t threads = 32 * warps;
     int bps = 0;
-    CK(solve_occupancy(threads, smem, &bps));
+    CK(solve_occupancy(W, threads, smem, &bps));
     if (bps < 1) return REI_ECUDA;
     grid = std::min<uint32_t>((uint32_t)(c->sm_count * bps), kMaxTeam);
     if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;

@@ -34,8 +34,8 @@ namespace rei {
 cudaError_t launch_stage(const StageJob *jobs_dev, uint32_t n_jobs, cudaStream_t stream);
 cudaError_t launch_solve(const SolveJob *job, uint32_t grid, uint32_t threads, size_t smem,
                          cudaStream_t stream);
-cudaError_t solve_occupancy(uint32_t threads, size_t smem, int *blocks_per_sm);
-cudaError_t solve_smem_max(size_t *bytes);
+cudaError_t solve_occupancy(uint32_t W, uint32_t threads, size_t smem, int *blocks_per_sm);
+cudaError_t solve_smem_max(uint32_t W, size_t *bytes);
 size_t solve_smem_bytes(uint32_t W, uint32_t n, uint32_t G, uint32_t max_len, uint32_t seg_cap,
                         bool gt_in_smem, uint32_t warps, uint32_t small_rows = 0);
 }  // namespace rei
@@ -302,7 +302,7 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     // launch shape (as the allocating path chooses it), within the dynamic
     // shared memory the search kernel can take
     size_t smem_max = 0;
-    NA_CK(solve_smem_max(&smem_max));
+    NA_CK(solve_smem_max(W, &smem_max));
     const uint32_t seg_cap = 2 * max_cost + 4;
     bool gt_smem = 4ull * (n + 1 + G + max_len + 2) <= 96 * 1024;
     uint32_t warps = 8;
@@ -322,7 +322,7 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     }
     if (smem > smem_max) NA_RET(REI_EINVAL);
     int bps = 0;
-    NA_CK(solve_occupancy(32 * warps, smem, &bps));
+    NA_CK(solve_occupancy(W, 32 * warps, smem, &bps));
     if (bps < 1) NA_RET(REI_ECUDA);
     const uint32_t grid = std::min<uint32_t>(kMaxTeam, (uint32_t)(prop.multiProcessorCount * bps));
 

@@ -8,8 +8,9 @@
 //   dedup     : table[2^k] of u64 slots = (fingerprint << 32) | index, where
 //               index < 2^31 is a cache row and PENDING|j marks chunk-local
 //               candidate j whose CS sits in tmp[j][W] until compaction
-//   chunk     : tmp[chunk][W], pending[chunk] (new slots), slotpos[chunk],
-//               bitmap[chunk/32] (survivors), blk[grid] (per-CTA counts)
+//   chunk     : tmp[chunk][W], bitmap[chunk/32] (marked candidates, then
+//               survivors), slotpos[chunk] (their slots), pending[chunk] (the
+//               survivors listed), blk[grid] (per-CTA counts)
 //   state     : SolveState (level, chunk position, counts, barrier, answer)
 #pragma once
 #include <cstdint>
@@ -120,7 +121,7 @@ struct SolveState {
     uint32_t otf;             // OnTheFly mode
     uint32_t partial_level;   // first level not completely cached
     unsigned long long found; // level-local index of the answer, or kNone
-    uint32_t pending_count;
+    uint32_t marked;          // the current chunk has marked candidates
     uint32_t ans_op, ans_l, ans_r, ans_cost;
     uint32_t tree_len;        // postfix tokens written
     uint64_t candidates;      // completed levels
