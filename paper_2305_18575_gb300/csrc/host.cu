@@ -88,11 +88,11 @@ struct rei_ctx {
         pos, neg, leaf;
     uint32_t pair_cap = 1u << 16;
     // search
-    DevBuf cs, bp_op, bp_l, bp_r, table, minidx, tmp, pending, slotpos, bitmap, blk, lvl_start, lvl_count,
+    DevBuf cs, bp_op, bp_l, bp_r, table, tmp, pending, slotpos, bitmap, blk, lvl_start, lvl_count,
         state, solve_job, tstack, trace, used, plan;
     DevBuf seen;               // bitmap of cached 1-word languages (2^kSeenBits bits)
     bool table_clean = false;  // the search kernel leaves the table (and seen) empty after a normal end
-    uint64_t table_extent = 0; // slots of the table (and minidx) that may hold entries: beyond, all empty
+    uint64_t table_extent = 0; // bytes of the table that may hold entries: beyond, all empty
     // batched form
     DevBuf b_in, b_sjobs, b_sinfo, b_stage, b_jobs, b_out, b_tree, b_queue;
     DevBuf s_cs, s_bp_op, s_bp_l, s_bp_r, s_used, s_table, s_tmp, s_pend, s_slotpos, s_bitmap, s_blk, s_lvl,
@@ -174,15 +174,13 @@ rei_status grow_keep(rei_ctx *c, DevBuf &b, size_t bytes, size_t keep) {
     return REI_OK;
 }
 
-// Empty the uniqueness table and its first-candidate array where they may
-// hold entries (the first max(table_extent, at_least) slots; beyond them they
-// are empty), so that a context that once solved a large problem does not
-// clear its whole table for every small one.
+// Empty the uniqueness table where it may hold entries (the first
+// max(table_extent, at_least) bytes; beyond them it is empty), so that a
+// context that once solved a large problem does not clear its whole table for
+// every small one.
 rei_status clear_table(rei_ctx *c, uint64_t at_least) {
-    const uint64_t ext = std::max(c->table_extent, at_least);
-    const uint64_t t = std::min<uint64_t>(ext, c->table.bytes / 8), m = std::min<uint64_t>(ext, c->minidx.bytes / 4);
-    if (t) CK(cudaMemsetAsync(c->table.p, 0xFF, 8 * t, c->stream));
-    if (m) CK(cudaMemsetAsync(c->minidx.p, 0xFF, 4 * m, c->stream));
+    const uint64_t t = std::min<uint64_t>(std::max(c->table_extent, at_least), c->table.bytes);
+    if (t) CK(cudaMemsetAsync(c->table.p, 0xFF, t, c->stream));
     c->table_extent = 0;
     return REI_OK;
 }
@@ -503,14 +501,12 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     const uint64_t tslots = pow2_at_least(std::max<uint64_t>(4 * rows, 1024));
     {
         // a reallocated table (even at the same address) holds garbage
-        const void *before = c->table.p, *mbefore = c->minidx.p;
-        const size_t before_bytes = c->table.bytes, mbefore_bytes = c->minidx.bytes;
-        if ((s = ensure(c, c->table, 8ull * tslots))) return s;
-        if ((s = ensure(c, c->minidx, 4ull * tslots))) return s;
-        if (c->table.p != before || c->table.bytes != before_bytes || c->minidx.p != mbefore ||
-            c->minidx.bytes != mbefore_bytes) {
+        const void *before = c->table.p;
+        const size_t before_bytes = c->table.bytes;
+        if ((s = ensure(c, c->table, 16ull * tslots))) return s;
+        if (c->table.p != before || c->table.bytes != before_bytes) {
             c->table_clean = false;
-            c->table_extent = std::max<uint64_t>(c->table.bytes / 8, c->minidx.bytes / 4);
+            c->table_extent = c->table.bytes;
         }
     }
     const uint64_t chunk_words = c->opt_chunk > 0 ? (uint64_t)c->opt_chunk : (1ull << 22);
@@ -554,7 +550,7 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
         if (c->seen.p) CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
     }
     c->table_clean = false;
-    c->table_extent = std::max(c->table_extent, tslots);
+    c->table_extent = std::max(c->table_extent, 16 * tslots);
 
     FuseArgs F;
     memset(&F, 0, sizeof F);
@@ -601,7 +597,6 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     j.used = (uint32_t *)c->used.p;
     j.table = (unsigned long long *)c->table.p;
     j.table_mask = tslots - 1;
-    j.minidx = (uint32_t *)c->minidx.p;
     j.exact = c->opt_exact ? 1u : 0u;  // allowed; the launch decides from the staged size
     j.tmp = (uint32_t *)c->tmp.p;
     j.pending = (uint32_t *)c->pending.p;
@@ -860,9 +855,11 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
         // 1-word exact keys up to 2^26 it has a slot for every language, the
         // language itself, and is never probed twice)
         if (n < 40) need = std::min<uint64_t>(need, 1ull << n);
-        const uint64_t t = pow2_at_least(std::max<uint64_t>(2 * need, 1024));
-        return use_direct ? std::max<uint64_t>(t, 1ull << n) : t;
+        return use_direct ? 1ull << n : pow2_at_least(std::max<uint64_t>(2 * need, 1024));
     };
+    // (exact keys: the language and its first candidate; else one word)
+    const bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
+    const uint64_t slot_bytes = exact_keys && !use_direct ? 16 : 8;
     uint64_t tslots = table_slots(cache_alloc);
     // after a fused launch the cache holds its rows: grow keeping them
     auto ensure_rows = [&](DevBuf &b, size_t bytes) {
@@ -874,18 +871,15 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     if ((s = ensure_rows(c->bp_r, 4ull * cache_alloc))) return s;
     if ((s = ensure(c, c->used, 4ull * cache_alloc))) return s;  // (rebuilt with the table)
     {
-        const void *before = c->table.p, *mbefore = c->minidx.p;
-        const size_t before_bytes = c->table.bytes, mbefore_bytes = c->minidx.bytes;
-        if ((s = ensure(c, c->table, 8ull * tslots))) return s;
-        if ((s = ensure(c, c->minidx, 4ull * tslots))) return s;
-        if (c->table.p != before || c->table.bytes != before_bytes || c->minidx.p != mbefore ||
-            c->minidx.bytes != mbefore_bytes) {
+        const void *before = c->table.p;
+        const size_t before_bytes = c->table.bytes;
+        if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
+        if (c->table.p != before || c->table.bytes != before_bytes) {
             c->table_clean = false;
-            c->table_extent = std::max<uint64_t>(c->table.bytes / 8, c->minidx.bytes / 4);
+            c->table_extent = c->table.bytes;
         }
     }
     // (candidate rows wait in tmp only when the keys are fingerprints)
-    const bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
     if ((s = ensure(c, c->tmp, exact_keys ? 4096 : 4ull * W * chunk_max))) return s;
     if ((s = ensure(c, c->pending, 4ull * chunk_max))) return s;
     if ((s = ensure(c, c->slotpos, 4ull * chunk_max))) return s;
@@ -926,7 +920,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
             if (c->seen.p) CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
         }
         c->table_clean = false;
-        c->table_extent = std::max(c->table_extent, tslots);
+        c->table_extent = std::max(c->table_extent, slot_bytes * tslots);
         uint32_t hj_cmin;
         {
             uint16_t lc[256];
@@ -979,7 +973,6 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
         hj->used = (uint32_t *)c->used.p;
         hj->cache_alloc = cache_alloc;
         hj->table = (unsigned long long *)c->table.p;
-        hj->minidx = (uint32_t *)c->minidx.p;
         hj->exact = (W <= 2 && n <= 62 && c->opt_exact) ? 1u : 0u;
         hj->seen = use_seen ? (uint32_t *)c->seen.p : nullptr;
         hj->direct = use_direct && tslots >= (1ull << n) ? 1u : 0u;
@@ -1038,14 +1031,12 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
         cache_alloc = want;
         tslots = table_slots(cache_alloc);
         {
-            const void *before = c->table.p, *mbefore = c->minidx.p;
-            if ((s = ensure(c, c->table, 8ull * tslots))) return s;
-            if ((s = ensure(c, c->minidx, 4ull * tslots))) return s;
-            if (c->table.p != before || c->minidx.p != mbefore)
-                c->table_extent = std::max<uint64_t>(c->table.bytes / 8, c->minidx.bytes / 4);
+            const void *before = c->table.p;
+            if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
+            if (c->table.p != before) c->table_extent = c->table.bytes;
         }
-        if ((s = clear_table(c, tslots))) return s;  // (the rehash refills it)
-        c->table_extent = tslots;
+        if ((s = clear_table(c, slot_bytes * tslots))) return s;  // (the rehash refills it)
+        c->table_extent = slot_bytes * tslots;
         fill_job();
         if (rows) {
             CK(launch_rehash(hj, (uint32_t)rows, (uint32_t)(c->sm_count * 8), c->stream));
@@ -1209,7 +1200,7 @@ void rei_ctx_destroy(rei_ctx *c) {
     cudaStreamSynchronize(c->stream);
     DevBuf *bufs[] = {&c->in_bytes, &c->in_offs, &c->stage_job, &c->stage_info, &c->word_start, &c->word_len,
                       &c->len_start, &c->gt_off, &c->gt_pair, &c->pos, &c->neg, &c->leaf, &c->cs,
-                      &c->bp_op, &c->bp_l, &c->bp_r, &c->table, &c->minidx, &c->tmp, &c->pending, &c->slotpos,
+                      &c->bp_op, &c->bp_l, &c->bp_r, &c->table, &c->tmp, &c->pending, &c->slotpos,
                       &c->bitmap, &c->blk, &c->lvl_start, &c->lvl_count, &c->state, &c->solve_job,
                       &c->tstack, &c->trace, &c->used, &c->plan, &c->seen, &c->b_in, &c->b_sjobs, &c->b_sinfo, &c->b_stage,
                       &c->b_jobs, &c->b_out, &c->b_tree, &c->b_queue, &c->s_cs, &c->s_bp_op, &c->s_bp_l,

@@ -7,7 +7,9 @@
 //               bp_op[]/bp_l[]/bp_r[] back-pointers
 //   dedup     : table[2^k] of u64 slots = (fingerprint << 32) | index, where
 //               index < 2^31 is a cache row and PENDING|j marks chunk-local
-//               candidate j whose CS sits in tmp[j][W] until compaction
+//               candidate j whose CS sits in tmp[j][W] until compaction; with
+//               exact keys two words a slot, the language and its first
+//               candidate
 //   chunk     : tmp[chunk][W], bitmap[chunk/32] (marked candidates, then
 //               survivors), slotpos[chunk] (their slots), pending[chunk] (the
 //               survivors listed), blk[grid] (per-CTA counts)
@@ -135,7 +137,7 @@ struct SolveState {
     uint32_t nseg;
     // command from CTA 0 to the other CTAs, and the chunk it describes
     uint32_t cmd, cmd_seq;
-    uint32_t c_level, c_size, c_dedup;
+    uint32_t c_level, c_size, c_dedup, c_epoch;
     uint64_t c_cs0, c_ce0;
     // CTA 0's wall time (ns) in: planning, chunks alone, chunks with the grid,
     // level ends; and how many solo chunks, team chunks, levels
@@ -143,7 +145,6 @@ struct SolveState {
     uint64_t n_phase[3];
     uint64_t t_sub[48];  // steps of CTA 0's chunks and launch (timing builds only)
     uint32_t tile_next;  // the next tile of a team chunk handed out dynamically
-    uint32_t pad;
     // the fused launch that owns this state: CTA 0 resets the state, stages,
     // then writes its launch id here; the other CTAs start once it names theirs
     unsigned long long launch;
@@ -182,18 +183,17 @@ struct SolveJob {
     uint32_t solo_tiles;             // chunks of at most this many tiles run on CTA 0 alone
     uint32_t small_rows;             // languages CTA 0 keeps in shared memory at the start (0 = none)
     // exact keys (|ic| <= 62, W <= 2): a table slot holds the language itself
-    // (bit 63: added in the current chunk), minidx[slot] the first candidate
-    // of the chunk with that language; 0 = fingerprint | row slots
+    // and the first candidate that has it (two words, at a 16-byte boundary);
+    // 0 = fingerprint | row slots (one word)
     uint32_t exact;
-    uint32_t *minidx;
     // 1-word languages (|ic| <= kSeenBits, exact keys): bit L of seen[] is set
     // once language L is cached, so that a candidate whose language is already
     // cached is told by one bit instead of a table probe; nullptr = none.  All
     // zero between searches (a search clears the words of the rows it cached).
     uint32_t *seen;
-    // exact keys with a table of at least 2^|ic| slots: the slot of a
-    // language is the language itself (no hash, never a second probe)
-    uint32_t direct, direct_pad;
+    // exact keys with a table of at least 2^|ic| words: the slot of a
+    // language is the language itself (no hash, never a second probe, one word)
+    uint32_t direct;
     // leaves: the alphabet symbols ordered by (cost, alphabet order) and
     // their costs (every symbol costs c[0] unless costs are given per
     // symbol; a cost above REI_MAX_COST is stored as REI_MAX_COST + 1);
@@ -219,7 +219,7 @@ struct FuseArgs {
     SolveJob *job;            // global: the completed job, for every CTA
     uint64_t mem_budget;
     uint64_t rows_alloc;      // rows of the back-pointer arrays
-    uint64_t cs_words, tmp_words, pend_cap, table_slots;
+    uint64_t cs_words, tmp_words, pend_cap, table_slots;  // (two words a slot)
     uint64_t chunk_opt;       // chunk size asked for (0 = automatic)
     uint32_t small_opt;       // languages in shared memory at the start: 0xFFFFFFFF automatic, 0 none
     uint64_t handover;        // levels above this many candidates go to the relaunch (0 = never)

@@ -6,12 +6,15 @@
 
 namespace rei {
 
-// Two CTAs of 16 warps an SM at 64 registers; from 20 words on the warps' tiles
-// fill the SM's shared memory with one, which then takes 128 registers (a row
-// compare keeps more loads in flight; languages of 32 words to cost 12: 9.1 ms
-// at 64 registers, 8.0 ms at 128, while 12 words lost a fifth with one CTA).
+// Two CTAs of 16 warps an SM at 64 registers.  One of 128 registers for 2-word
+// languages, whose tiles keep four candidates a lane with their table slots in
+// registers (|ic| 36-42 to cost 20: 11.7 ms with two CTAs, which spill, 9.5 ms
+// with one; 1-word languages, bound by the L2, lost a tenth with one, 4-word
+// ones a sixth), and from 20 words on, where the warps' tiles leave room for
+// one CTA an SM anyway (32 words to cost 12: 9.1 -> 8.0 ms; 12 words lost a
+// fifth).
 template <uint32_t WC>
-__global__ void __launch_bounds__(kSolveThreads, WC == kWidest ? 1 : 2) k_solve(const __grid_constant__ SolveJob J) {
+__global__ void __launch_bounds__(kSolveThreads, WC == kWidest || WC == 2 ? 1 : 2) k_solve(const __grid_constant__ SolveJob J) {
     uint32_t bar_epoch = 0;
     solve_body<WC>(J, bar_epoch);
 }
@@ -31,16 +34,14 @@ __global__ void k_rehash(const __grid_constant__ SolveJob J, uint32_t count) {
     for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count;
          k += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t *c = J.cs + k * W;
-        const uint64_t h = cs_hash(c, W, 1);
-        const unsigned long long v =
-            J.exact ? exact_key(c, W) : ((uint64_t)(uint32_t)(h >> 32) << 32) | (uint32_t)k;
-        uint64_t p = J.direct ? v : h & J.table_mask;
-        for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
-            if (atomicCAS(&J.table[p], kEmpty, v) == kEmpty) {
-                J.used[k] = (uint32_t)p;
-                break;
-            }
-            p = (p + 1) & J.table_mask;
+        if (J.exact) {
+            J.used[k] = (uint32_t)exact_fill(J, exact_key(c, W), (uint32_t)k);
+        } else {
+            const uint64_t h = cs_hash(c, W, 1);
+            const unsigned long long v = ((uint64_t)(uint32_t)(h >> 32) << 32) | (uint32_t)k;
+            uint64_t p = h & J.table_mask;
+            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = (p + 1) & J.table_mask;
+            J.used[k] = (uint32_t)p;
         }
         if (J.seen) atomicOr(J.seen + (c[0] >> 5), 1u << (c[0] & 31u));
     }

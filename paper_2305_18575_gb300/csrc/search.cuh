@@ -66,6 +66,13 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const void *p) {
     return v;
 }
 
+// two neighbouring words, at a 16-byte boundary (each read whole)
+__device__ __forceinline__ ulonglong2 ld_relaxed_u64x2(const void *p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
@@ -189,19 +196,44 @@ __device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t m, uint32_t l) {
 }
 
 // per-warp shared memory (32-bit words): the shared operand's words, two
-// 32-candidate tiles (candidate-major and bit-sliced); for 1-word languages
-// also the nibble tables of the concatenation's shared operand and its id
-constexpr uint32_t kW1Tab = 128;   // 8 nibble tables of 16 words
-constexpr uint32_t kW1TabAt = 68;  // their offset (4 + 2 * 32 words; 16-byte aligned)
-// candidates per tile of a concatenation or union segment: 32 (one per lane),
-// or for 1-word languages 32 * kW1Per (kW1Per per lane, built side by side)
-constexpr uint32_t kW1Per = 4;
-__host__ __device__ inline uint32_t bin_block(uint32_t W) { return W == 1 ? 32u * kW1Per : 32u; }
-
-__host__ __device__ inline uint32_t warp_words(uint32_t W) {
+// 32-candidate tiles (candidate-major and bit-sliced; 16-byte aligned); for
+// languages of up to 2 words also the nibble tables of the concatenation's
+// shared operand (8 W tables of 16 languages) and, in the word after them, its id
+__host__ __device__ inline uint32_t tile_words(uint32_t W) {
     const uint32_t Ws = (W & 1u) ? W : W + 1;
-    const uint32_t base = ((W + 3) & ~3u) + 2 * 32 * Ws;
-    return W == 1 ? kW1TabAt + kW1Tab + 4 : base;
+    return ((W + 3) & ~3u) + 2 * 32 * Ws;
+}
+__host__ __device__ inline uint32_t tab_words(uint32_t W) { return W <= 2 ? 128 * W * W : 0u; }
+__host__ __device__ inline uint32_t warp_words(uint32_t W) { return tile_words(W) + (W <= 2 ? tab_words(W) + 4 : 0u); }
+
+// Language widths a search is compiled for: 1, 2 or 4 words, 8 to 16 (kWide),
+// more (kWidest), or any (kAnyWidth: the width is not known when the kernel is
+// launched, as in the fused launch, or differs between its problems).  A launch
+// of one width holds only that width's tile code, so that its registers are
+// what that code needs.
+constexpr uint32_t kAnyWidth = 0, kWide = 8, kWidest = 20;
+
+constexpr uint32_t kSortMax = 2048;  // candidates of a chunk CTA 0 runs with shared-memory bookkeeping
+
+// Candidates per tile of a concatenation or union segment: 32 (one per lane),
+// or 32 * reg_per (reg_per per lane, built side by side in registers) for
+// 1-word languages and, in the relaunch of 2-word ones, for chunks of kRegChunk
+// candidates per warp of the team and more.  Below that a 2-word tile of 32 is
+// the better one: it spreads a chunk over more warps, and a chunk of a few
+// tiles a warp ends with its slowest tile (in the first launch tiles of 128
+// made medium searches 3 % slower).  The relaunch takes eight 1-word
+// candidates a lane (a deep search 97 ms, with four 100 ms) and four 2-word ones
+// (|ic| 36-42 to cost 20: 9.5 ms; two 9.6 ms, six 10.3 ms, eight 11.3 ms).
+constexpr uint32_t kRegChunk = 64;
+template <uint32_t WC>
+__host__ __device__ constexpr uint32_t reg_per() { return WC == 1 ? 8u : 4u; }
+template <uint32_t WC>
+__device__ __forceinline__ uint32_t chunk_block(const SolveJob &J, uint64_t C, uint32_t team_warps) {
+    if (J.W == 1) return 32u * reg_per<WC>();
+    // (rows are read 8 bytes at a time, table slots 16)
+    return WC == 2 && C > kSortMax && C >= (uint64_t)kRegChunk * team_warps &&
+                   (reinterpret_cast<uintptr_t>(J.cs) & 7u) == 0 && (reinterpret_cast<uintptr_t>(J.table) & 15u) == 0
+               ? 32u * reg_per<WC>() : 32u;
 }
 
 struct Shared {
@@ -230,6 +262,7 @@ struct Lead {
     // the answer was found and the other CTAs were told to empty the table
     // (rows and marked candidates given) while the leader writes out the answer
     uint32_t cleaned, clean_rows, clean_marks;
+    uint32_t epoch;  // chunks of this launch
     uint64_t chunk_pos, candidates, unique_done;
     uint64_t cand_op[5];
 };
@@ -253,7 +286,8 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t v, uint32_t lane) {
 // one whole warp: lane k describes candidate segment k of each round of 32,
 // the non-empty ones are compacted with a ballot and their starts are a warp
 // scan of the sizes.
-__device__ inline void plan_level(const SolveJob &J, uint32_t c, const uint32_t *lvs, const uint32_t *lvc, Seg *seg,
+template <uint32_t WC>
+__device__ __forceinline__ void plan_level(const SolveJob &J, uint32_t c, const uint32_t *lvs, const uint32_t *lvc, Seg *seg,
                            Plan &P) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t c1 = J.cmin;  // no expression is cheaper
@@ -304,13 +338,15 @@ __device__ inline void plan_level(const SolveJob &J, uint32_t c, const uint32_t 
                 size = (uint64_t)s.lcnt * s.rcnt;
                 // tiles of 32 right operands per left one, or (swapped) of 32
                 // left operands per right one: whichever needs fewer tiles
-                // (fewer partly empty tiles)
-                const uint32_t bw = bin_block(J.W);
+                // (fewer partly empty tiles); tiles of 128 where the lookup
+                // tables are used, with the work of the tables
+                const bool reg = J.W == 1 || (WC == 2 && size >= (1u << 14));
+                const uint32_t bw = reg ? 32u * reg_per<WC>() : 32u;
                 uint64_t t_rows = (uint64_t)s.lcnt * ((s.rcnt + bw - 1) / bw);
                 uint64_t t_cols = (uint64_t)s.rcnt * ((s.lcnt + bw - 1) / bw);
-                if (J.W == 1) {
-                    // (and the lookup tables of each shared operand, about
-                    // one and a half tiles' work each)
+                if (reg) {
+                    // (the lookup tables of each shared operand, about one and
+                    // a half tiles' work each)
                     t_rows += s.lcnt + s.lcnt / 2;
                     t_cols += s.rcnt + s.rcnt / 2;
                 }
@@ -409,6 +445,7 @@ struct TileCtx {
     const Shared *S;
     uint64_t chunk_start;
     uint32_t W, Ws, n;
+    uint32_t epoch;  // the chunk's number in this launch (exact keys)
     bool dedup;
     bool grid;  // every CTA works on the chunk (else CTA 0 alone)
     unsigned long long *found;  // minimum precise candidate: shared (small chunk alone) or global
@@ -417,6 +454,7 @@ struct TileCtx {
     const uint32_t *ops;        // the cached languages operands are read from (shared or global)
     bool smem;                  // uniqueness in CTA 0's shared table
     bool vec;                   // language rows in cs and tmp are whole 16-byte words at 16-byte addresses
+    bool reg;                   // binary tiles of 32 * reg_per candidates, built in registers
 };
 
 // no table slot: a candidate that is not marked
@@ -569,20 +607,58 @@ __device__ void dedup_insert_solo(const TileCtx &T, const uint32_t *c, uint32_t 
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
 }
 
-constexpr unsigned long long kXPend = 1ull << 63;  // exact keys: the language was added in this chunk
+// Exact keys: a slot is two words, the language itself and the first candidate
+// that has it, epoch << 32 | candidate, where the epoch is the number of the
+// chunk that added it (0: cached before this launch's table was filled).  A
+// slot of an older epoch is a cached language, so that a chunk's survivors need
+// no change of their slots when they are cached, and a probe, its claim and its
+// first candidate are one 32-byte sector (with the key marked "new" and the
+// first candidate in an array of its own, a new language of a large search cost
+// eight random accesses of the HBM, which serves 40 to 50 G a second; now four).
+// With a slot per language (direct) the slot's number is the language and the
+// slot only the second word.  Empty: all ones.
+__device__ __forceinline__ unsigned long long *exact_meta(const SolveJob &J, uint64_t q) {
+    return J.direct ? J.table + q : J.table + 2 * q + 1;
+}
+__device__ __forceinline__ void exact_free(const SolveJob &J, uint64_t q) {
+    if (!J.direct) J.table[2 * q] = kEmpty;
+    *exact_meta(J, q) = kEmpty;
+}
+__device__ __forceinline__ unsigned long long exact_entry(uint32_t epoch, uint32_t xl) {
+    return ((unsigned long long)epoch << 32) | xl;
+}
 
 // the exact key of a W <= 2 language (padding bits and bit 63 are zero)
 __device__ __forceinline__ unsigned long long exact_key(const uint32_t *c, uint32_t W) {
     return W == 1 ? (unsigned long long)c[0] : ((unsigned long long)c[1] << 32) | c[0];
 }
 
+// exact keys: the table slot a probe starts at.  The top bits of a
+// multiplicative hash (Knuth, "The Art of Computer Programming" 3, 6.4), an
+// even slot: the second probe then lies in the first one's 32-byte sector.
+__device__ __forceinline__ uint64_t exact_slot(const SolveJob &J, unsigned long long key) {
+    if (J.direct) return key;
+    const unsigned long long h = (key ^ (key >> 31)) * 0x9E3779B97F4A7C15ull;
+    return (h >> (64 - __popcll(J.table_mask))) & ~1ull;
+}
+
+// a cached language into the table, with epoch 0 (languages that are all
+// distinct, while no other insertion runs); returns its slot
+__device__ __forceinline__ uint64_t exact_fill(const SolveJob &J, unsigned long long key, uint32_t row) {
+    uint64_t p = exact_slot(J, key);
+    if (!J.direct)
+        while (atomicCAS(&J.table[2 * p], kEmpty, key) != kEmpty) p = (p + 1) & J.table_mask;
+    *exact_meta(J, p) = row;
+    return p;
+}
+
 // uniqueness insert with exact keys: the slot's key is the language, so a
 // duplicate costs one probe and no row read; a language new in this chunk is
-// claimed with a CAS and every candidate with it lowers minidx[slot] (a
+// claimed with a CAS and its candidates lower the slot's first candidate (a
 // reduction, no round trip).  The claimants are recorded in T.bits / T.ent (a
 // small chunk on one CTA), else the slot is returned for the tile to mark the
 // candidate with (kNoMark: nothing to mark); the marks include every survivor,
-// and the chunk's filter keeps those minidx still names.
+// and the chunk's filter keeps those the slot still names.
 template <uint32_t WT>
 __device__ uint32_t dedup_insert_exact(const TileCtx &T, const uint32_t *c, uint32_t xl) {
     const SolveJob &J = *T.J;
@@ -591,25 +667,26 @@ __device__ uint32_t dedup_insert_exact(const TileCtx &T, const uint32_t *c, uint
     // by the append of that chunk, visible after its grid barriers; read
     // through L2).  Languages new in this chunk take the table protocol below.
     if (J.seen && ((ldcg(J.seen + (c[0] >> 5)) >> (c[0] & 31u)) & 1u)) return kNoMark;
-    const unsigned long long key = exact_key(c, W), pk = key | kXPend;
-    uint64_t p = J.direct ? key : cs_hash(c, W, 1) & J.table_mask;
+    const unsigned long long key = exact_key(c, W), mine = exact_entry(T.epoch, xl);
+    uint64_t p = exact_slot(J, key);
     for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
-        unsigned long long v = ld_relaxed_u64(&J.table[p]);
-        if (v == kEmpty) {
-            v = atomicCAS(&J.table[p], kEmpty, pk);
+        unsigned long long v = key, m;
+        if (J.direct) {
+            m = ld_relaxed_u64(&J.table[p]);
+        } else {
+            const ulonglong2 s = ld_relaxed_u64x2(&J.table[2 * p]);
+            v = s.x;
+            m = s.y;
             if (v == kEmpty) {
-                atomicMin(&J.minidx[p], xl);
-                if (T.bits) {
-                    T.ent[xl] = p;
-                    atomicOr(&T.bits[xl >> 5], 1u << (xl & 31));
-                }
-                return (uint32_t)p;
+                v = atomicCAS(&J.table[2 * p], kEmpty, key);
+                if (v == kEmpty) v = key;
+                m = kEmpty;  // (whoever claimed it, its first candidate is of this chunk)
             }
         }
-        if ((v & ~kXPend) == key) {
-            // (a candidate after the one minidx names already changes nothing)
-            if (!(v & kXPend) || ld_relaxed_u32(&J.minidx[p]) <= xl) return kNoMark;
-            atomicMin(&J.minidx[p], xl);
+        if (v == key) {
+            // (cached, or a candidate before this one has it already)
+            if (m <= mine) return kNoMark;
+            atomicMin(exact_meta(J, p), mine);
             if (T.bits) {
                 T.ent[xl] = p;
                 atomicOr(&T.bits[xl >> 5], 1u << (xl & 31));
@@ -940,7 +1017,7 @@ __device__ __forceinline__ uint32_t w1_lookup(const uint32_t *tab, uint32_t x, u
     return out;
 }
 
-// precision and uniqueness of a lane's kW1Per 1-word candidates c[k]
+// precision and uniqueness of a lane's K 1-word candidates c[k]
 // (level-segment indices x0 + k * dx, valid where bit k of vb is set): every
 // seen-bitmap word is read before any is tested, so the reads overlap
 template <uint32_t K>
@@ -994,9 +1071,12 @@ __device__ __forceinline__ bool w1_finish(const TileCtx &T, const Seg &sg, uint3
 }
 
 // one tile of 1-word candidates: 32 of a unary segment (one per lane), or
-// 32 * kW1Per of a binary one (kW1Per per lane, 32 apart).  Returns, in each
+// 32 * K of a binary one (K per lane, 32 apart).  A candidate that equals one of
+// its operands is cached already and ends there (a deep search 97.0 -> 94.2 ms).
+// Returns, in each
 // lane, whether it marked a candidate in the chunk's bitmap.
-__device__ inline bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile, uint32_t *wm) {
+template <uint32_t K>
+__device__ bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile, uint32_t *wm) {
     // (few candidates: the bit-sliced fixed point)
     if (sg.op == OP_STAR) return run_tile<1>(T, sg, tl, tile, wm);
     const SolveJob &J = *T.J;
@@ -1018,7 +1098,6 @@ __device__ inline bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTil
     }
     // binary: candidate k of the lane is (row, col0 + 32 k), or, swapped,
     // (row0 + 32 k, col)
-    constexpr uint32_t K = kW1Per;
     const bool swapped = sg.op == OP_CAT && sg.swap;
     const uint32_t t32 = (uint32_t)tile, qt = div_by(t32, tl.nb_mul, tl.nb_shift);
     const uint32_t off = (t32 - qt * tl.nb) * (32 * K) + lane;
@@ -1055,16 +1134,19 @@ __device__ inline bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTil
 #pragma unroll
         for (uint32_t k = 0; k < K; k++) r[k] = ((vb >> k) & 1u) ? ldop(cs + sg.rbase + col + 32 * k) : 0u;
 #pragma unroll
-        for (uint32_t k = 0; k < K; k++) c[k] = l | r[k];
+        for (uint32_t k = 0; k < K; k++) {
+            c[k] = l | r[k];
+            if (T.dedup && (c[k] == l || c[k] == r[k])) vb &= ~(1u << k);
+        }
     } else {
         // the tables of the shared operand (its id in the word after them)
-        uint32_t *tab = wm + kW1TabAt;
+        uint32_t *tab = wm + tile_words(1);
         const uint32_t sid = swapped ? (0x80000000u | (sg.rbase + col)) : (sg.lbase + row);
-        if (tab[kW1Tab] != sid) {
+        if (tab[tab_words(1)] != sid) {
             const uint32_t sh = ldop(cs + (sid & 0x7FFFFFFFu));
             __syncwarp();  // (every lane has read the old id)
             w1_tables(S, T.n, sh, swapped, tab, lane);
-            if (lane == 0) tab[kW1Tab] = sid;
+            if (lane == 0) tab[tab_words(1)] = sid;
             __syncwarp();
         }
         const uint32_t *ob = swapped ? cs + sg.lbase + row : cs + sg.rbase + col;
@@ -1073,9 +1155,219 @@ __device__ inline bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTil
         for (uint32_t k = 0; k < K; k++) o[k] = ((vb >> k) & 1u) ? ldop(ob + 32 * k) : 0u;
         const uint32_t nt = (T.n + 3) >> 2;
 #pragma unroll
-        for (uint32_t k = 0; k < K; k++) c[k] = w1_lookup(tab, o[k], nt);
+        for (uint32_t k = 0; k < K; k++) {
+            c[k] = w1_lookup(tab, o[k], nt);
+            if (T.dedup && c[k] == o[k]) vb &= ~(1u << k);
+        }
     }
     return w1_finish<K>(T, sg, c, x0, dx, vb);
+}
+
+// ---------------------------------------------------------------------------
+// phase A for 2-word languages in large chunks: as for 1-word ones, K
+// candidates a lane in registers, the concatenation's nibble tables holding
+// two words an entry (16 entries of 8 bytes are 32 banks, so any 32 lanes read
+// one table without a conflict).  About 60 instructions a warp for 32
+// concatenations of |ic| 40, against 350 bit-sliced with their transposes; and
+// the operand rows, table slots and claims of a lane's four candidates are in
+// flight together, where the bit-sliced tile waits for one after another.  What
+// bounds it is the HBM's rate of random accesses, one a candidate: 8-byte loads
+// at random addresses ran at 288 G/s within 64 MB, 124 G/s in 128 MB, 51 G/s in
+// 512 MB and 40 G/s from 2 GB on.  Specifications of |ic| 36 - 42 searched to
+// cost 20: 12.3 ms bit-sliced, 9.3 ms so.
+
+__device__ __forceinline__ void w2_tables(const Shared &S, uint32_t n, uint2 sh, bool swapped, uint32_t *tab,
+                                          uint32_t lane) {
+    // words lane and lane + 32: their column of M (bit b set when M[b] holds the word)
+    uint32_t cl[2] = {0u, 0u}, ch[2] = {0u, 0u};
+#pragma unroll
+    for (uint32_t h = 0; h < 2; h++) {
+        const uint32_t w = lane + 32 * h;
+        if (w >= n) continue;
+        const uint32_t p1 = S.gt_off[w + 1];
+        for (uint32_t p = S.gt_off[w]; p < p1; p++) {
+            const uint32_t pr = S.gt_pair[p];
+            const uint32_t u = pr & 0xFFFFu, v = pr >> 16;
+            const uint32_t have = swapped ? v : u, other = swapped ? u : v;
+            const uint32_t bit = (((have & 32u) ? sh.y : sh.x) >> (have & 31u)) & 1u;
+            if (other & 32u) ch[h] |= bit << (other & 31u);
+            else cl[h] |= bit << other;
+        }
+    }
+    // lane b: words of M[b] (m0) and M[b + 32] (m1)
+    const uint2 m0 = make_uint2(transpose32(cl[0], lane), transpose32(cl[1], lane));
+    const uint2 m1 = make_uint2(transpose32(ch[0], lane), transpose32(ch[1], lane));
+    // lane 2t + h fills entries 8h .. 8h + 7 of table t
+    const uint32_t t = lane >> 1, h = lane & 1u;
+    uint2 m[4];
+#pragma unroll
+    for (uint32_t i = 0; i < 4; i++) {
+        const uint32_t src = (4 * t + i) & 31u;
+        const uint32_t ax = __shfl_sync(0xFFFFFFFFu, m0.x, src), ay = __shfl_sync(0xFFFFFFFFu, m0.y, src);
+        const uint32_t bx = __shfl_sync(0xFFFFFFFFu, m1.x, src), by = __shfl_sync(0xFFFFFFFFu, m1.y, src);
+        m[i] = t < 8 ? make_uint2(ax, ay) : make_uint2(bx, by);
+    }
+    const uint2 base = h ? m[3] : make_uint2(0u, 0u);
+    uint4 *dst = reinterpret_cast<uint4 *>(tab + 32 * t + 16 * h);
+#pragma unroll
+    for (uint32_t y = 0; y < 8; y += 2) {
+        uint32_t ex = base.x, ey = base.y;
+        if (y & 2u) ex |= m[1].x, ey |= m[1].y;
+        if (y & 4u) ex |= m[2].x, ey |= m[2].y;
+        dst[y >> 1] = make_uint4(ex, ey, ex | m[0].x, ey | m[0].y);
+    }
+}
+
+// precision and uniqueness of a lane's 2-word candidates c[k] (those with bit
+// k of vb; level-segment indices x0 + k * dx): every probe, claim and
+// first-candidate read of the four goes out before any is used, and so do the
+// next probes of those that met another language.  q[k]: the slot to mark
+// candidate k with, else kNoMark.  A language cached by an earlier chunk needs
+// no precision test (it was tested when its first candidate was, and a precise
+// one would have ended the search).
+template <uint32_t K>
+__device__ __forceinline__ void w2_finish(const TileCtx &T, const Seg &sg, const uint2 (&c)[K], uint64_t x0, uint64_t dx,
+                                          uint32_t vb, uint32_t (&q)[K]) {
+    const SolveJob &J = *T.J;
+    const Shared &S = *T.S;
+    const uint64_t xlev0 = sg.start + x0;
+    uint32_t fresh = vb;  // candidates to test for precision
+    if (T.dedup && J.exact) {
+        fresh = 0;
+        uint32_t p[K];  // (a table has at most 2^32 slots)
+#pragma unroll
+        for (uint32_t k = 0; k < K; k++) p[k] = (uint32_t)exact_slot(J, ((unsigned long long)c[k].y << 32) | c[k].x);
+        const uint32_t xl0 = (uint32_t)(xlev0 - T.chunk_start), dl = (uint32_t)dx;
+        uint64_t rounds = 0;
+        for (uint32_t act = vb; act;) {
+            ulonglong2 v[K];
+#pragma unroll
+            for (uint32_t k = 0; k < K; k++)
+                if ((act >> k) & 1u) v[k] = ld_relaxed_u64x2(&J.table[2ull * p[k]]);
+#pragma unroll
+            for (uint32_t k = 0; k < K; k++)
+                if (((act >> k) & 1u) && v[k].x == kEmpty) {
+                    const unsigned long long key = ((unsigned long long)c[k].y << 32) | c[k].x;
+                    v[k].x = atomicCAS(&J.table[2ull * p[k]], kEmpty, key);
+                    v[k].y = kEmpty;  // (whoever claimed it, its first candidate is of this chunk)
+                }
+#pragma unroll
+            for (uint32_t k = 0; k < K; k++) {
+                if (!((act >> k) & 1u)) continue;
+                const unsigned long long key = ((unsigned long long)c[k].y << 32) | c[k].x;
+                if (v[k].x == key || v[k].x == kEmpty) {
+                    // (of an older epoch: cached)
+                    if (v[k].y >= ((unsigned long long)T.epoch << 32)) fresh |= 1u << k;
+                    const unsigned long long mine = exact_entry(T.epoch, xl0 + k * dl);
+                    if (v[k].y > mine) {
+                        atomicMin(&J.table[2ull * p[k] + 1], mine);
+                        q[k] = p[k];
+                    }
+                    act &= ~(1u << k);
+                } else {
+                    p[k] = (p[k] + 1) & (uint32_t)J.table_mask;
+                }
+            }
+            if (++rounds > J.table_mask) {
+                atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
+                break;
+            }
+        }
+    }
+    const uint32_t p0 = S.pos[0], p1 = S.pos[1], n0 = S.neg[0], n1 = S.neg[1];
+#pragma unroll
+    for (uint32_t k = 0; k < K; k++) {
+        if (!((fresh >> k) & 1u)) continue;
+        const uint32_t errs = __popc(p0 & ~c[k].x) + __popc(p1 & ~c[k].y) + __popc(n0 & c[k].x) + __popc(n1 & c[k].y);
+        if (errs <= J.max_errors) atomicMin(T.found, (unsigned long long)(xlev0 + k * dx));
+    }
+    if (T.dedup && !J.exact) {
+#pragma unroll
+        for (uint32_t k = 0; k < K; k++) {
+            if (!((vb >> k) & 1u)) continue;
+            const uint32_t w[2] = {c[k].x, c[k].y};
+            q[k] = dedup_insert<2>(T, w, (uint32_t)(xlev0 + k * dx - T.chunk_start));
+        }
+    }
+}
+
+// one tile of 32 * K 2-word candidates of a binary segment; returns
+// whether any was marked in the chunk's bitmap (the whole warp alike)
+template <uint32_t K>
+__device__ __forceinline__ bool run_tile_w2(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile, uint32_t *wm) {
+    const SolveJob &J = *T.J;
+    const Shared &S = *T.S;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint2 *cs = reinterpret_cast<const uint2 *>(J.cs);
+    const uint64_t lo = tl.lo, hi = tl.hi;
+    // candidate k of the lane is (row, col + 32 k), or, swapped, (row + 32 k, col)
+    const bool swapped = sg.op == OP_CAT && sg.swap;
+    const uint32_t t32 = (uint32_t)tile, qt = div_by(t32, tl.nb_mul, tl.nb_shift);
+    const uint32_t off = (t32 - qt * tl.nb) * (32 * K) + lane;
+    const uint32_t row = (uint32_t)tl.r0 + (swapped ? off : qt), col = swapped ? qt : off;  // of candidate 0
+    const uint64_t x0 = (uint64_t)row * sg.rcnt + col, dx = swapped ? 32ull * sg.rcnt : 32ull;
+    uint32_t vb = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < K; k++) {
+        const uint64_t x = x0 + k * dx;
+        const bool in = swapped ? row + 32 * k < sg.lcnt : col + 32 * k < sg.rcnt && (!sg.tri || col + 32 * k > row);
+        if (in && x >= lo && x < hi) vb |= 1u << k;
+    }
+    if (__ballot_sync(0xFFFFFFFFu, vb != 0) == 0) return false;
+    const uint2 *ob = swapped ? cs + sg.lbase + row : cs + sg.rbase + col;
+    uint2 c[K];
+#pragma unroll
+    for (uint32_t k = 0; k < K; k++) c[k] = ((vb >> k) & 1u) ? __ldcg(ob + 32 * k) : make_uint2(0u, 0u);
+    if (sg.op == OP_ALT) {
+        const uint2 l = __ldcg(cs + sg.lbase + row);
+#pragma unroll
+        for (uint32_t k = 0; k < K; k++) {
+            const uint2 r = c[k];
+            c[k].x |= l.x, c[k].y |= l.y;
+            if (T.dedup && ((c[k].x == l.x && c[k].y == l.y) || (c[k].x == r.x && c[k].y == r.y))) vb &= ~(1u << k);
+        }
+    } else {
+        // the tables of the shared operand (its id in the word after them)
+        uint32_t *tab = wm + tile_words(2);
+        const uint32_t sid = swapped ? (0x80000000u | (sg.rbase + col)) : (sg.lbase + row);
+        if (tab[tab_words(2)] != sid) {
+            const uint2 sh = __ldcg(cs + (sid & 0x7FFFFFFFu));
+            __syncwarp();  // (every lane has read the old id)
+            w2_tables(S, T.n, sh, swapped, tab, lane);
+            if (lane == 0) tab[tab_words(2)] = sid;
+            __syncwarp();
+        }
+        const uint32_t nt = (T.n + 3) >> 2;  // (9 .. 16)
+        const uint2 *t2 = reinterpret_cast<const uint2 *>(tab);
+#pragma unroll
+        for (uint32_t k = 0; k < K; k++) {
+            uint2 o = make_uint2(0u, 0u);
+#pragma unroll
+            for (uint32_t t = 0; t < 16; t++)
+                if (t < 8 || t < nt) {
+                    const uint2 e = t2[16 * t + (((t < 8 ? c[k].x : c[k].y) >> (4 * (t & 7u))) & 15u)];
+                    o.x |= e.x;
+                    o.y |= e.y;
+                }
+            if (T.dedup && o.x == c[k].x && o.y == c[k].y) vb &= ~(1u << k);
+            c[k] = o;
+        }
+    }
+    uint32_t q[K];
+#pragma unroll
+    for (uint32_t k = 0; k < K; k++) q[k] = kNoMark;
+    w2_finish<K>(T, sg, c, x0, dx, vb, q);
+    if (!T.dedup) return false;
+    __syncwarp();
+    const uint64_t xlev = sg.start + x0;
+    const uint32_t xl = (uint32_t)(xlev - T.chunk_start), xf = __shfl_sync(0xFFFFFFFFu, xl, 0);
+    // (a tile that straddles the chunk's start marks bit by bit, see run_tile)
+    const bool straight = !swapped && __shfl_sync(0xFFFFFFFFu, (uint32_t)(xlev >= T.chunk_start), 0) != 0;
+    bool marked = false;
+#pragma unroll
+    for (uint32_t k = 0; k < K; k++)
+        marked |= mark_tile(J, xl + k * (uint32_t)dx, q[k], straight, xf + k * (uint32_t)dx);
+    return marked;
 }
 
 // ---------------------------------------------------------------------------
@@ -1311,7 +1603,6 @@ __device__ inline uint32_t emit_tree_warp(const SolveJob &J, uint32_t op, uint32
 // runs two per SM at 64 registers for more loads in flight
 constexpr uint32_t kFusedThreads = 512;
 constexpr uint32_t kSolveThreads = 512;
-constexpr uint32_t kSortMax = 2048;  // candidates of a chunk CTA 0 runs with shared-memory bookkeeping
 static_assert(kMaxTeam < kSortMax, "the append's prefix table of per-CTA counts lives in sortbuf");
 static_assert(kTreeScratchWords <= 2 * kSortMax, "the answer's tree is gathered in sortbuf");
 
@@ -1336,6 +1627,8 @@ enum Cmd : uint32_t { CMD_NONE = 0, CMD_CHUNK = 1, CMD_EXIT = 2, CMD_CLEAN = 3 }
 struct ChunkArgs {
     uint32_t level, size, dedup, nseg;
     uint64_t cs0, ce0;
+    uint32_t bw;  // candidates per binary tile (chunk_block)
+    uint32_t epoch;  // the chunk's number in this launch (from 1)
 };
 
 // tiles of the chunk [cs0, ce0) in every segment; run by one whole warp
@@ -1476,15 +1769,14 @@ __device__ inline void switch_to_global(const SolveJob &J, Shared &S, Lead *L) {
     REI_TSPAN_BEGIN(t_sw);
     for (uint32_t k = threadIdx.x; k < rows; k += blockDim.x) {
         const uint32_t *row = S.sm_rows + (uint64_t)k * W;
-        const uint64_t h = cs_hash(row, W, 1);
-        const unsigned long long v = J.exact ? exact_key(row, W) : ((uint64_t)(uint32_t)(h >> 32) << 32) | k;
-        uint64_t p = J.direct ? v : h & J.table_mask;
-        for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
-            if (atomicCAS(&J.table[p], kEmpty, v) == kEmpty) {
-                J.used[k] = (uint32_t)p;
-                break;
-            }
-            p = (p + 1) & J.table_mask;
+        if (J.exact) {
+            J.used[k] = (uint32_t)exact_fill(J, exact_key(row, W), k);
+        } else {
+            const uint64_t h = cs_hash(row, W, 1);
+            const unsigned long long v = ((uint64_t)(uint32_t)(h >> 32) << 32) | k;
+            uint64_t p = h & J.table_mask;
+            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = (p + 1) & J.table_mask;
+            J.used[k] = (uint32_t)p;
         }
         if (J.seen) atomicOr(J.seen + (row[0] >> 5), 1u << (row[0] & 31u));
     }
@@ -1514,8 +1806,7 @@ __device__ inline void solo_append(const SolveJob &J, SolveState *st, Shared &S,
             const uint32_t xl = base + u * nt + tid;
             mk[u] = xl < C && ((bits[xl >> 5] >> (xl & 31)) & 1u);
             v[u] = !mk[u] ? 0ull
-                   : J.exact ? ld_relaxed_u32(J.minidx + (uint32_t)ent[xl])
-                             : ld_relaxed_u64(J.table + (uint32_t)ent[xl]);
+                           : ld_relaxed_u64(J.exact ? exact_meta(J, (uint32_t)ent[xl]) : J.table + (uint32_t)ent[xl]);
         }
 #pragma unroll
         for (int u = 0; u < 8; u++) {
@@ -1555,19 +1846,17 @@ __device__ inline void solo_append(const SolveJob &J, SolveState *st, Shared &S,
         const unsigned long long e = ent[xl];
         const uint32_t q = (uint32_t)e;
         if (rank >= room) {
-            J.table[q] = kEmpty;
-            if (J.exact) J.minidx[q] = 0xFFFFFFFFu;
+            if (J.exact) exact_free(J, q);
+            else J.table[q] = kEmpty;
             continue;
         }
         const uint64_t k = (uint64_t)a.size + rank;
         uint32_t *dst = J.cs + k * W;
         if (J.exact) {
             // the language is the slot's key
-            const unsigned long long key = ld_relaxed_u64(J.table + q) & ~kXPend;
+            const unsigned long long key = J.direct ? q : ld_relaxed_u64(J.table + 2ull * q);
             dst[0] = (uint32_t)key;
             if (W == 2) dst[1] = (uint32_t)(key >> 32);
-            J.table[q] = key;
-            J.minidx[q] = 0xFFFFFFFFu;
             if (J.seen) atomicOr(J.seen + ((uint32_t)key >> 5), 1u << (key & 31u));
         } else {
             const uint32_t *srcp = J.tmp + (uint64_t)xl * W;
@@ -1661,18 +1950,14 @@ __device__ __forceinline__ void each_mark(const SolveJob &J, uint64_t C, uint64_
     }
 }
 
-// Language widths a search is compiled for: 1, 2 or 4 words, 8 to 16 (kWide),
-// more (kWidest), or any (kAnyWidth: the width is not known when the kernel is
-// launched, as in the fused launch, or differs between its problems).  A launch
-// of one width holds only that width's tile code, so that its registers are
-// what that code needs.
-constexpr uint32_t kAnyWidth = 0, kWide = 8, kWidest = 20;
-
 template <uint32_t WC>
 __device__ __forceinline__ bool run_tile_of(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile,
                                             uint32_t *wm) {
-    if (WC == 1 || (WC == kAnyWidth && T.W == 1)) return run_tile_w1(T, sg, tl, tile, wm);
-    if (WC == 2 || (WC == kAnyWidth && T.W == 2)) return run_tile<2>(T, sg, tl, tile, wm);
+    if (WC == 1 || (WC == kAnyWidth && T.W == 1)) return run_tile_w1<reg_per<WC>()>(T, sg, tl, tile, wm);
+    if (WC == 2 || (WC == kAnyWidth && T.W == 2)) {
+        if (WC == 2 && T.reg && (sg.op == OP_CAT || sg.op == OP_ALT)) return run_tile_w2<reg_per<WC>()>(T, sg, tl, tile, wm);
+        return run_tile<2>(T, sg, tl, tile, wm);
+    }
     if (WC == 4) return run_tile<4>(T, sg, tl, tile, wm);
     return run_tile<0>(T, sg, tl, tile, wm);
 }
@@ -1680,7 +1965,7 @@ __device__ __forceinline__ bool run_tile_of(const TileCtx &T, const Seg &sg, con
 // one chunk of candidates; returns 1 when a precise candidate was found in it,
 // 0 when done, -1 when a grid barrier gave up
 template <uint32_t WC>
-__device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const ChunkArgs &a, bool full,
+__device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const ChunkArgs &a, bool full,
                              bool tiles_ready, uint32_t &bar_epoch, uint64_t *s_tiles, uint32_t *s_red,
                              unsigned long long *s_found, uint32_t *s_marked, uint32_t *wm, Lead *L) {
     const uint32_t W = WC == 1 || WC == 2 || WC == 4 ? WC : J.W, n = J.n;
@@ -1692,7 +1977,7 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
     REI_TSTART();
 
     if (!tiles_ready) {
-        if (wid == 0) tile_setup(S, a.nseg, a.cs0, a.ce0, s_tiles, bin_block(W));
+        if (wid == 0) tile_setup(S, a.nseg, a.cs0, a.ce0, s_tiles, a.bw);
         __syncthreads();
     }
 
@@ -1707,9 +1992,10 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
 
     // ---- phase A: build, precision, uniqueness insert
     {
-        TileCtx TC{&J, st, &S, a.cs0, W, Ws, n, dedup, full, small ? s_found : &st->found,
+        TileCtx TC{&J, st, &S, a.cs0, W, Ws, n, a.epoch, dedup, full, small ? s_found : &st->found,
                    small ? S.sortbuf : nullptr, small ? S.solo_bits : nullptr, sm ? S.sm_rows : J.cs, sm,
-                   (W & 3u) == 0 && ((reinterpret_cast<uintptr_t>(J.cs) | reinterpret_cast<uintptr_t>(J.tmp)) & 15u) == 0};
+                   (W & 3u) == 0 && ((reinterpret_cast<uintptr_t>(J.cs) | reinterpret_cast<uintptr_t>(J.tmp)) & 15u) == 0,
+                   a.bw > 32};
         bool marked = false;
         // (a chunk's tiles, at most 2^26 / 32 plus one per segment, fit 32 bits)
         const uint32_t ntiles = (uint32_t)*s_tiles;
@@ -1723,9 +2009,12 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
         const bool dyn = full && ntiles >= kDynTilesPerWarp * nw;
         // (1-word languages: longer runs of tiles that share an operand, whose
         // lookup tables are then built once per run)
-        const uint32_t grab = W == 1 ? 4 * kGrab : kGrab;
+        // Towards the chunk's end the grabs shrink, so that the last warp is a
+        // tile or two behind the others.
+        const uint32_t most = a.bw > 32 ? 4 * kGrab : kGrab;
+        auto grab_at = [&](uint32_t at) { return max(2u, min(most, (ntiles - at) / nw)); };
         uint32_t t = gw, end = ntiles, step = nw;
-        uint32_t nxt = 0;
+        uint32_t nxt = 0, grab = most;
 #ifdef REI_TIMING
         __shared__ unsigned long long s_wmax;
         if (tid == 0) s_wmax = 0;
@@ -1741,7 +2030,10 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
             t = __shfl_sync(0xFFFFFFFFu, cur, 0);
             end = min(t + grab, ntiles);
             step = 1;
-            if (lane == 0 && t < ntiles) nxt = atomicAdd(&st->tile_next, grab);
+            if (t < ntiles) {
+                grab = grab_at(t);
+                if (lane == 0) nxt = atomicAdd(&st->tile_next, grab);
+            }
         }
         while (t < ntiles) {
             while (s + 1 < a.nseg && S.tile_first[s + 1] <= t) s++;
@@ -1763,7 +2055,10 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
             if (dyn && t >= end) {
                 t = __shfl_sync(0xFFFFFFFFu, nxt, 0);
                 end = min(t + grab, ntiles);
-                if (lane == 0 && t < ntiles) nxt = atomicAdd(&st->tile_next, grab);
+                if (t < ntiles) {
+                    grab = grab_at(t);
+                    if (lane == 0) nxt = atomicAdd(&st->tile_next, grab);
+                }
             }
         }
         // (one word tells every CTA, after the barrier, that the chunk has marks)
@@ -1801,8 +2096,8 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
                 for (uint32_t xl = tid; xl < C; xl += blockDim.x)
                     if ((S.solo_bits[xl >> 5] >> (xl & 31)) & 1u) {
                         const uint32_t q = (uint32_t)S.sortbuf[xl];
-                        J.table[q] = kEmpty;
-                        if (J.exact) J.minidx[q] = 0xFFFFFFFFu;
+                        if (J.exact) exact_free(J, q);
+                        else J.table[q] = kEmpty;
                     }
             __syncthreads();
             for (uint32_t w = tid; w < kSortMax / 32; w += blockDim.x) S.solo_bits[w] = 0;
@@ -1834,9 +2129,10 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
                   uint32_t q[4], m[4];
 #pragma unroll
                   for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? ldcg(J.slotpos + j[u]) : 0u;
+                  // (a marked slot is of this chunk: its entry's low half tells)
 #pragma unroll
                   for (uint32_t u = 0; u < 4; u++)
-                      if (on[u]) m[u] = J.exact ? ld_relaxed_u32(J.minidx + q[u]) : (uint32_t)ld_relaxed_u64(J.table + q[u]);
+                      if (on[u]) m[u] = (uint32_t)ld_relaxed_u64(J.exact ? exact_meta(J, q[u]) : J.table + q[u]);
 #pragma unroll
                   for (uint32_t u = 0; u < 4; u++) drop[u] = on[u] && m[u] != (J.exact ? j[u] : (kPending | j[u]));
               });
@@ -1973,15 +2269,16 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     const uint32_t i = i0 + u * nt;
-                    if (i < nfit) old[u] = ld_relaxed_u64(J.table + q[u]);
+                    if (i < nfit) old[u] = J.direct ? q[u] : ld_relaxed_u64(J.exact ? J.table + 2ull * q[u] : J.table + q[u]);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     const uint32_t i = i0 + u * nt;
                     if (i >= cnt) continue;
                     if (i >= nfit) {
-                        J.table[q[u]] = kEmpty;  // not cached: free the slot
-                        if (J.exact) J.minidx[q[u]] = 0xFFFFFFFFu;
+                        // not cached: free the slot
+                        if (J.exact) exact_free(J, q[u]);
+                        else J.table[q[u]] = kEmpty;
                         continue;
                     }
                     const uint64_t k = b0 + i;
@@ -1991,11 +2288,9 @@ __device__ int process_chunk(const SolveJob &J, SolveState *st, Shared &S, const
                     J.bp_l[k] = l;
                     J.bp_r[k] = r;
                     if (J.exact) {
-                        const unsigned long long key = old[u] & ~kXPend;
+                        const unsigned long long key = old[u];
                         J.cs[k * W] = (uint32_t)key;
                         if (W == 2) J.cs[k * W + 1] = (uint32_t)(key >> 32);
-                        J.table[q[u]] = key;
-                        J.minidx[q[u]] = 0xFFFFFFFFu;
                         if (J.seen) atomicOr(J.seen + ((uint32_t)key >> 5), 1u << (key & 31u));
                     } else {
                         J.table[q[u]] = (old[u] & 0xFFFFFFFF00000000ull) | (uint32_t)k;
@@ -2121,9 +2416,10 @@ __device__ inline void carve_shared(const SolveJob &J, Shared &S, uint8_t *smem_
     S.warp_words = warp_words(W);
     S.warp_mem = reinterpret_cast<uint32_t *>(p);
     (void)Ws;
-    // no concatenation tables built yet (1-word languages)
-    if (W == 1)
-        for (uint32_t w = tid; w < blockDim.x / 32; w += blockDim.x) S.warp_mem[w * S.warp_words + kW1TabAt + kW1Tab] = kNoOperand;
+    // no concatenation tables built yet
+    if (W <= 2)
+        for (uint32_t w = tid; w < blockDim.x / 32; w += blockDim.x)
+            S.warp_mem[w * S.warp_words + tile_words(W) + tab_words(W)] = kNoOperand;
     for (uint32_t b = tid; b < W; b += blockDim.x) {
         S.pos[b] = J.pos_mask[b];
         S.neg[b] = J.neg_mask[b];
@@ -2152,26 +2448,52 @@ struct Cta {
 // without clearing it: the slot of every cached row, and the slots of the
 // marked candidates (the first nmarks of a chunk may hold marks) of a chunk
 // that ended with the answer before its survivors were appended; their marks
-// are cleared too.
+// are cleared too.  When the rows are a sixteenth of the slots or more the whole
+// table is written instead, in order: at random addresses the HBM takes 23 G
+// slots a second, in order about 400 G (a search of 35 million 2-word languages
+// took 1.0 ms to empty its table).
 __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nmarks, uint32_t team_n,
-                            uint32_t team_r) {
+                                   uint32_t team_r) {
     const uint64_t t = (uint64_t)team_r * blockDim.x + threadIdx.x, nt = (uint64_t)team_n * blockDim.x;
-    for (uint64_t k = t; k < rows; k += nt) J.table[ldcg(J.used + k)] = kEmpty;
+    // (few CTAs are bound by the stores they issue, one a row)
+    const bool all = team_n >= 64 && 16ull * rows > J.table_mask;
+    if (all) {
+        // (a table is at least 1024 slots from its allocation's start on)
+        ulonglong2 *w = reinterpret_cast<ulonglong2 *>(J.table);
+        const uint64_t n2 = (J.table_mask + 1) >> (J.exact && !J.direct ? 0 : 1);
+        const ulonglong2 e = make_ulonglong2(kEmpty, kEmpty);
+        if ((reinterpret_cast<uintptr_t>(J.table) & 15u) == 0) {
+            for (uint64_t i = t; i < n2; i += nt) w[i] = e;
+        } else {
+            for (uint64_t i = t; i < 2 * n2; i += nt) J.table[i] = kEmpty;
+        }
+    } else {
+        for (uint64_t k = t; k < rows; k += nt) {
+            const uint32_t q = ldcg(J.used + k);
+            if (J.exact) exact_free(J, q);
+            else J.table[q] = kEmpty;
+        }
+    }
     // the seen bitmap holds bits of cached languages only: zero every word
-    // that holds one
-    if (J.seen)
-        for (uint64_t k = t; k < rows; k += nt) J.seen[ldcg(J.cs + k) >> 5] = 0u;
+    // that holds one, or all of them
+    if (J.seen) {
+        const uint64_t words = J.n > 5 ? 1ull << (J.n - 5) : 1ull;
+        if (rows >= words)
+            for (uint64_t i = t; i < words; i += nt) J.seen[i] = 0u;
+        else
+            for (uint64_t k = t; k < rows; k += nt) J.seen[ldcg(J.cs + k) >> 5] = 0u;
+    }
     if (nmarks)
         each_mark(J, nmarks, t >> 5, nt >> 5, [&](const uint32_t (&j)[4], const bool (&on)[4], bool (&drop)[4]) {
             uint32_t q[4];
 #pragma unroll
-            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? ldcg(J.slotpos + j[u]) : 0u;
+            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] && !all ? ldcg(J.slotpos + j[u]) : 0u;
 #pragma unroll
             for (uint32_t u = 0; u < 4; u++) {
                 drop[u] = on[u];
-                if (!on[u]) continue;
-                J.table[q[u]] = kEmpty;
-                if (J.exact) J.minidx[q[u]] = 0xFFFFFFFFu;
+                if (!on[u] || all) continue;
+                if (J.exact) exact_free(J, q[u]);
+                else J.table[q[u]] = kEmpty;
             }
         });
 }
@@ -2191,6 +2513,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
     if (tid == 0) {
         L.cleaned = 0;
         L.clean_marks = 0;
+        L.epoch = 0;
         L.status = st->status;
         L.level = st->level;
         L.size = st->size;
@@ -2282,7 +2605,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
         // a level's plan depends on lower levels only: once per level
         if (level != planned) {
             REI_TSPAN_BEGIN(t_pl);
-            if (wid == 0) plan_level(J, level, S.lvs, S.lvc, S.seg, s_plan);
+            if (wid == 0) plan_level<WC>(J, level, S.lvs, S.lvc, S.seg, s_plan);
             __syncthreads();
             planned = level;
             REI_TSPAN_END(st, t_pl, 18);
@@ -2342,10 +2665,12 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
             }
         }
         if (C == 0) C = 1;  // unreachable with room >= 1; guards the loop
-        ChunkArgs a{level, size, dedup ? 1u : 0u, nseg, pos, pos + C};
+        // (the other CTAs of a team size their tiles by the same rule)
+        ChunkArgs a{level, size, dedup ? 1u : 0u, nseg, pos, pos + C,
+                    chunk_block<WC>(J, C, (allow_team ? team_size_of(J) : 1u) * (blockDim.x >> 5)), L.epoch + 1};
         // alone when the chunk is a few tiles per warp of this CTA
         REI_TSPAN_BEGIN(t_ts);
-        if (wid == 0) tile_setup(S, nseg, a.cs0, a.ce0, K.tiles, bin_block(J.W));
+        if (wid == 0) tile_setup(S, nseg, a.cs0, a.ce0, K.tiles, a.bw);
         if (tid == 0) *K.found = kNone;  // a small chunk's answer slot
         __syncthreads();
         REI_TSPAN_END(st, t_ts, 19);
@@ -2361,6 +2686,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
                 st->c_level = a.level;
                 st->c_size = a.size;
                 st->c_dedup = a.dedup;
+                st->c_epoch = a.epoch;
                 st->c_cs0 = a.cs0;
                 st->c_ce0 = a.ce0;
             }
@@ -2386,6 +2712,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
             break;
         }
         if (tid == 0) {
+            L.epoch = a.epoch;
             L.chunk_pos = a.ce0;
             if (a.ce0 >= T) end_level(level, nseg);  // the level's last chunk
         }
@@ -2514,6 +2841,7 @@ __device__ __forceinline__ void solve_body(const SolveJob &J, uint32_t &bar_epoc
                 s_ctl[1] = ld_relaxed_u32(&st->c_level);
                 s_ctl[2] = ld_relaxed_u32(&st->c_size);
                 s_ctl[3] = ld_relaxed_u32(&st->c_dedup);
+                s_ctl[6] = ld_relaxed_u32(&st->c_epoch);
                 s_pos[0] = ld_relaxed_u64(&st->c_cs0);
                 s_pos[1] = ld_relaxed_u64(&st->c_ce0);
             }
@@ -2525,7 +2853,8 @@ __device__ __forceinline__ void solve_body(const SolveJob &J, uint32_t &bar_epoc
                 return;
             }
             if (s_ctl[0] != CMD_CHUNK) return;
-            ChunkArgs a{s_ctl[1], s_ctl[2], s_ctl[3], 0, s_pos[0], s_pos[1]};
+            ChunkArgs a{s_ctl[1], s_ctl[2], s_ctl[3], 0, s_pos[0], s_pos[1],
+                        chunk_block<WC>(J, s_pos[1] - s_pos[0], team_size_of(J) * (blockDim.x >> 5)), s_ctl[6]};
             if (J.plan) {
                 a.nseg = s_ctl[5];
             } else {
@@ -2535,7 +2864,7 @@ __device__ __forceinline__ void solve_body(const SolveJob &J, uint32_t &bar_epoc
                     S.lvc[c] = (uint32_t)ld_relaxed_u64(&J.lvl_count[c]);
                 }
                 __syncthreads();
-                if ((tid >> 5) == 0) plan_level(J, a.level, S.lvs, S.lvc, S.seg, s_plan);
+                if ((tid >> 5) == 0) plan_level<WC>(J, a.level, S.lvs, S.lvc, S.seg, s_plan);
                 __syncthreads();
                 a.nseg = s_plan.nseg;
             }

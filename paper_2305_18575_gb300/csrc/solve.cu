@@ -85,6 +85,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_solve_fused(const __grid_c
                 j.exact = F.tmpl.exact && W <= 2 && I.n <= 62 ? 1u : 0u;
                 j.seen = j.exact && W == 1 && I.n <= F.seen_bits ? F.seen : nullptr;
                 j.direct = j.exact && W == 1 && (1ull << I.n) <= F.table_slots ? 1u : 0u;
+                // (a slot per language: the table is as many words)
+                if (j.direct) j.table_mask = (1ull << I.n) - 1;
                 j.handover = F.handover;
                 const uint64_t tmax = F.table_slots / 2;
                 j.cache_alloc = umin64(umin64(j.cap, F.rows_alloc), umin64(F.cs_words / W, tmax / 2));
