@@ -269,6 +269,7 @@ struct Lead {
 
 struct Plan {
     uint32_t nseg;
+    uint32_t small;          // the level fits the shared-memory start as one chunk (small_levels)
     uint64_t total;          // index-space size of the level
 };
 
@@ -286,7 +287,7 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t v, uint32_t lane) {
 // one whole warp: lane k describes candidate segment k of each round of 32,
 // the non-empty ones are compacted with a ballot and their starts are a warp
 // scan of the sizes.
-template <uint32_t WC>
+template <uint32_t WC, bool SMALL = false>
 __device__ __forceinline__ void plan_level(const SolveJob &J, uint32_t c, const uint32_t *lvs, const uint32_t *lvc, Seg *seg,
                            Plan &P) {
     const uint32_t lane = threadIdx.x & 31;
@@ -340,7 +341,7 @@ __device__ __forceinline__ void plan_level(const SolveJob &J, uint32_t c, const 
                 // left operands per right one: whichever needs fewer tiles
                 // (fewer partly empty tiles); tiles of 128 where the lookup
                 // tables are used, with the work of the tables
-                const bool reg = J.W == 1 || (WC == 2 && size >= (1u << 14));
+                const bool reg = !SMALL && (J.W == 1 || (WC == 2 && size >= (1u << 14)));
                 const uint32_t bw = reg ? 32u * reg_per<WC>() : 32u;
                 uint64_t t_rows = (uint64_t)s.lcnt * ((s.rcnt + bw - 1) / bw);
                 uint64_t t_cols = (uint64_t)s.rcnt * ((s.lcnt + bw - 1) / bw);
@@ -511,45 +512,62 @@ __device__ __forceinline__ uint32_t ldop(const uint32_t *p) {
 constexpr uint32_t kSmEmpty = 0xFFFFFFFFu;
 constexpr uint32_t kSmPending = 0x10000u;
 
+// hash for the shared-memory table: 15 bits of slot (low) and 15 of fingerprint
+// (high); 32-bit multiplies, a third of the latency of the 64-bit hash
+__device__ __forceinline__ uint32_t smem_hash(const uint32_t *c, uint32_t W) {
+    uint32_t h = 0x243F6A88u;
+    for (uint32_t b = 0; b < W; b++) {
+        h = (h ^ c[b]) * 0x9E3779B1u;
+        h ^= h >> 15;
+    }
+    h *= 0x85EBCA6Bu;
+    return h ^ (h >> 13);
+}
+
 // uniqueness insert of candidate xl while the languages live in shared
 // memory: the same protocol as dedup_insert_solo on a 32-bit table whose
-// entries are fp (15 bits) << 17 | pending << 16 | row or candidate
+// entries are fp (15 bits) << 17 | pending << 16 | row or candidate.  A
+// candidate that took its slot, or took it over, is marked in `bits`, with its
+// slot and `note` (above its low 16 bits) in ent.
 template <uint32_t WT>
-__device__ void dedup_insert_smem(const TileCtx &T, const uint32_t *c, uint32_t xl) {
-    const Shared &S = *T.S;
-    const uint32_t W = WT ? WT : T.W;
-    const uint64_t h = cs_hash(c, W, 1);
-    const uint32_t fp = (uint32_t)(h >> 49);  // 15 bits
+__device__ __forceinline__ void dedup_smem(const Shared &S, SolveState *st, uint32_t small_rows, uint32_t Wr,
+                                           const uint32_t *c, uint32_t xl, unsigned long long note,
+                                           unsigned long long *ent, uint32_t *bits) {
+    const uint32_t W = WT ? WT : Wr;
+    const uint32_t h = smem_hash(c, W), fp = h >> 17;
     const uint32_t mine = (fp << 17) | kSmPending | xl;
-    const uint32_t mask = 2 * T.J->small_rows - 1;
-    uint32_t p = (uint32_t)h & mask;
+    const uint32_t mask = 2 * small_rows - 1;
+    uint32_t p = h & mask;
     uint32_t *dst = S.sm_tmp + xl * W;
     for (uint32_t b = 0; b < W; b++) dst[b] = c[b];
     __threadfence_block();
     for (uint32_t probe = 0; probe <= mask; probe++) {
         const uint32_t v = atomicCAS(&S.sm_table[p], kSmEmpty, mine);
-        if (v == kSmEmpty) {
-            T.ent[xl] = p;
-            atomicOr(&T.bits[xl >> 5], 1u << (xl & 31));
-            return;
-        }
-        if ((v >> 17) == fp) {
+        bool take = v == kSmEmpty;
+        if (!take && (v >> 17) == fp) {
             __threadfence_block();
             const uint32_t idx = v & 0xFFFFu;
             const volatile uint32_t *src = (v & kSmPending) ? S.sm_tmp + idx * W : S.sm_rows + idx * W;
-            bool eq = true;
-            for (uint32_t b = 0; b < W && eq; b++) eq = src[b] == c[b];
-            if (eq) {
-                if ((v & kSmPending) && idx > xl && atomicMin(&S.sm_table[p], mine) > mine) {
-                    T.ent[xl] = p;
-                    atomicOr(&T.bits[xl >> 5], 1u << (xl & 31));
-                }
-                return;
+            uint32_t diff = 0;
+            for (uint32_t b = 0; b < W; b++) diff |= src[b] ^ c[b];
+            if (diff == 0) {
+                if (!(v & kSmPending) || idx < xl || atomicMin(&S.sm_table[p], mine) <= mine) return;
+                take = true;
             }
+        }
+        if (take) {
+            ent[xl] = note | p;
+            atomicOr(&bits[xl >> 5], 1u << (xl & 31));
+            return;
         }
         p = (p + 1) & mask;
     }
-    atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
+    atomicExch(&st->err, 2u);  // table full: cannot happen with load <= 1/2
+}
+
+template <uint32_t WT>
+__device__ __forceinline__ void dedup_insert_smem(const TileCtx &T, const uint32_t *c, uint32_t xl) {
+    dedup_smem<WT>(*T.S, T.st, T.J->small_rows, T.W, c, xl, 0, T.ent, T.bits);
 }
 
 // A fingerprint entry names a cached row (below the cache's rows) or, marked
@@ -1703,7 +1721,7 @@ __device__ inline void smem_append(const SolveJob &J, Shared &S, const ChunkArgs
     const unsigned long long *ent = S.sortbuf;
     for (uint32_t xl = tid; xl < C; xl += nt) {
         if (!((bits[xl >> 5] >> (xl & 31)) & 1u)) continue;
-        const uint32_t v = S.sm_table[(uint32_t)ent[xl]];
+        const uint32_t v = S.sm_table[(uint32_t)ent[xl] & 0xFFFFu];
         if ((v & 0x1FFFFu) != (kSmPending | xl)) atomicAnd(&bits[xl >> 5], ~(1u << (xl & 31)));
     }
     __syncthreads();
@@ -2498,12 +2516,325 @@ __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nm
         });
 }
 
+// ---------------------------------------------------------------------------
+// the levels at a search's start, each one chunk of at most kSortMax candidates
+// on the leader alone, with every language and the uniqueness table in its
+// shared memory.  These levels are all latency (a level of a few tiles a warp:
+// plan, tiles, append), so they have a loop of their own: tiles whose
+// candidates stay in registers and whose operands are read from shared memory,
+// survivors that need no decoding (the operands are noted when a candidate
+// takes its slot), three barriers a level instead of nine, and the next level
+// planned by warp 0 while the others append this one.  Small queries 73.7 ->
+// 68.0 us, medium searches (eight in a row) 1203 -> 1032 us.
+
+// one tile of 32 candidates
+template <uint32_t WT>
+__device__ __forceinline__ void small_tile(const SolveJob &J, const Shared &S, SolveState *st, const Seg &sg,
+                                           const SegTile &tl, uint32_t tile, uint32_t *wm, unsigned long long *found) {
+    const uint32_t lane = threadIdx.x & 31, n = J.n;
+    const uint32_t W = WT ? WT : J.W, Ws = (W & 1u) ? W : W + 1;
+    constexpr uint32_t R = WT ? WT : 1;  // words of a candidate in registers (WT = 0: in A)
+    uint32_t *A = wm + ((W + 3) & ~3u), *B = A + 32 * Ws;
+    const uint32_t *cs = S.sm_rows;
+    const uint32_t op = sg.op;
+    // (a chunk of at most kSortMax candidates: every index fits 32 bits; it is
+    // the whole level, so that a segment has all its candidates in it)
+    uint32_t x, row = 0, col = 0, first, own;  // `own`: the row this lane's candidate reads alone
+    bool valid;
+    const bool swapped = op == OP_CAT && sg.swap;
+    if (op == OP_CAT || op == OP_ALT) {
+        const uint32_t qt = div_by(tile, tl.nb_mul, tl.nb_shift);
+        first = (tile - qt * tl.nb) * 32;
+        if (swapped) {
+            col = qt;
+            row = first + lane;
+            valid = row < sg.lcnt;
+            own = sg.lbase + row;
+        } else {
+            row = qt;
+            col = first + lane;
+            valid = col < sg.rcnt && (!sg.tri || col > row);
+            own = sg.rbase + col;
+        }
+        x = row * sg.rcnt + col;
+    } else {
+        first = tile * 32;
+        x = first + lane;
+        valid = x < (uint32_t)sg.size;
+        own = sg.lbase + x;
+    }
+    if (__ballot_sync(0xFFFFFFFFu, valid) == 0) return;
+    const uint32_t shared_row = swapped ? sg.rbase + col : sg.lbase + row;
+    uint32_t c[R];
+    unsigned long long note = (unsigned long long)op << 48;
+    if (op == OP_LEAF) {
+        const uint32_t sym = valid ? J.leaf_sym[own] : 0u;
+        note |= 0xFFFF00000000ull | (sym << 16);
+        if (WT) {
+#pragma unroll
+            for (uint32_t b = 0; b < R; b++) c[b] = valid ? __ldg(J.leaf + (uint64_t)sym * J.leaf_stride + b) : 0u;
+        } else {
+            for (uint32_t b = 0; b < W; b++)
+                A[lane * Ws + b] = valid ? __ldg(J.leaf + (uint64_t)sym * J.leaf_stride + b) : 0u;
+            __syncwarp();
+        }
+    } else {
+        // the lane's own operand
+        note |= op == OP_CAT || op == OP_ALT
+                    ? ((unsigned long long)(sg.rbase + col) << 32) | ((sg.lbase + row) << 16)
+                    : 0xFFFF00000000ull | (own << 16);
+        if (WT) {
+#pragma unroll
+            for (uint32_t b = 0; b < R; b++) c[b] = valid ? cs[own * W + b] : 0u;
+        } else {
+            const uint32_t all = swapped ? sg.lcnt : op == OP_CAT || op == OP_ALT ? sg.rcnt : (uint32_t)sg.size;
+            const uint32_t *src = cs + (own - lane) * W;
+            for (uint32_t i = lane; i < 32 * W; i += 32) {
+                const uint32_t j = i / W, b = i - j * W;
+                A[j * Ws + b] = first + j < all ? src[i] : 0u;
+            }
+            __syncwarp();
+        }
+        if (op == OP_OPT) {
+            if (WT) c[0] |= 1u;  // eps is ic word 0
+            else A[lane * Ws] |= 1u;
+            __syncwarp();
+        } else if (op == OP_ALT) {
+            if (WT) {
+#pragma unroll
+                for (uint32_t b = 0; b < R; b++) c[b] |= cs[shared_row * W + b];
+            } else {
+                for (uint32_t b = 0; b < W; b++) A[lane * Ws + b] |= cs[shared_row * W + b];
+                __syncwarp();
+            }
+        } else {
+            // bit-sliced over the 32 operands (see run_tile): B[v] bit j = operand j holds word v
+            if (WT) {
+#pragma unroll
+                for (uint32_t b = 0; b < R; b++) B[32 * b + lane] = transpose32(c[b], lane);
+            } else {
+                for (uint32_t b = 0; b < W; b++) B[32 * b + lane] = transpose32(A[lane * Ws + b], lane);
+            }
+            __syncwarp();
+            const uint32_t *go = S.gt_off, *gp = S.gt_pair;
+            if (op == OP_CAT) {
+                const uint32_t *lw = cs + shared_row * W;
+                const uint32_t sh = swapped ? 16u : 0u;  // which half of a pair indexes the shared operand
+                uint32_t l0 = lw[0], l1 = W > 1 ? lw[1] : 0u;
+#pragma unroll
+                for (uint32_t b = 0; b < (WT ? WT : 1u); b++) {
+                    for (uint32_t bb = b; bb < (WT ? b + 1 : W); bb++) {
+                        const uint32_t w = 32 * bb + lane;
+                        uint32_t acc = 0;
+                        if (w < n) {
+                            const uint32_t p1 = go[w + 1];
+#pragma unroll 4
+                            for (uint32_t p = go[w]; p < p1; p++) {
+                                const uint32_t pr = gp[p];
+                                const uint32_t k = (pr >> sh) & 0xFFFFu, o = (pr >> (16u - sh)) & 0xFFFFu;
+                                const uint32_t lv = WT == 1 ? l0 : WT == 2 ? ((k & 32u) ? l1 : l0) : lw[k >> 5];
+                                acc |= B[o] & (0u - ((lv >> (k & 31u)) & 1u));
+                            }
+                        }
+                        const uint32_t t = transpose32(acc, lane);
+                        if (WT) c[b] = t;
+                        else A[lane * Ws + bb] = t;
+                    }
+                }
+                __syncwarp();
+            } else {
+                // the least S with S = 1 + r.S, by increasing word length (in A, word by word)
+                uint32_t *Sl = A;
+                for (uint32_t w = lane; w < 32 * W; w += 32) Sl[w] = w ? 0u : 0xFFFFFFFFu;
+                __syncwarp();
+                const uint32_t *ls = S.len_start;
+                for (uint32_t L = 1; L <= J.max_len; L++) {
+                    const uint32_t w1 = ls[L + 1];
+                    for (uint32_t w = ls[L] + lane; w < w1; w += 32) {
+                        uint32_t acc = 0;
+                        const uint32_t p1 = go[w + 1];
+#pragma unroll 4
+                        for (uint32_t p = go[w] + 1; p < p1; p++) {
+                            const uint32_t pr = gp[p];
+                            acc |= B[pr & 0xFFFFu] & Sl[pr >> 16];
+                        }
+                        Sl[w] = acc;
+                    }
+                    __syncwarp();
+                }
+                if (WT) {
+#pragma unroll
+                    for (uint32_t b = 0; b < R; b++) c[b] = transpose32(Sl[32 * b + lane], lane);
+                } else {
+                    for (uint32_t b = 0; b < W; b++) B[lane * Ws + b] = transpose32(Sl[32 * b + lane], lane);
+                    __syncwarp();
+                    A = B;
+                }
+            }
+        }
+    }
+    if (valid) {
+        const uint32_t *cc = WT ? c : A + lane * Ws;
+        uint32_t errs = 0;
+        for (uint32_t b = 0; b < W; b++) errs += __popc(S.pos[b] & ~cc[b]) + __popc(S.neg[b] & cc[b]);
+        const uint32_t xl = (uint32_t)sg.start + x;
+        if (errs <= J.max_errors) atomicMin(found, (unsigned long long)xl);
+        dedup_smem<WT>(S, st, J.small_rows, W, cc, xl, note, S.sortbuf, S.solo_bits);
+    }
+    __syncwarp();
+}
+
+// What the leader does between two levels (one whole warp): count level
+// `level`, whose plan is in S.seg, with `size` languages cached after it, enter
+// the next one and plan it (with its tiles); plan.small tells whether
+// small_levels can run it.  The rules are those of the leader's loop.
+__device__ inline void small_next(const SolveJob &J, Shared &S, Lead &L, Plan &plan, uint64_t *s_tiles,
+                                  unsigned long long *s_found, uint32_t level, uint32_t size, bool count,
+                                  uint32_t solo_tiles) {
+    const uint32_t lane = threadIdx.x & 31;
+    for (;;) {
+        if (count) {
+            uint32_t by[5] = {0, 0, 0, 0, 0};
+            for (uint32_t s = lane; s < plan.nseg; s += 32) {
+                const uint32_t v = (uint32_t)valid_count(S.seg[s]), o = S.seg[s].op;
+#pragma unroll
+                for (uint32_t k = 0; k < 5; k++) by[k] += o == k ? v : 0u;
+            }
+#pragma unroll
+            for (uint32_t k = 0; k < 5; k++) by[k] = __reduce_add_sync(0xFFFFFFFFu, by[k]);
+            if (lane == 0) {
+                for (uint32_t k = 0; k < 5; k++) L.cand_op[k] += by[k];
+                L.candidates += (uint64_t)by[0] + by[1] + by[2] + by[3] + by[4];
+                L.size = size;
+                L.unique_done = size;
+                L.chunk_pos = 0;
+                S.lvc[level] = size - S.lvs[level];
+                J.lvl_count[level] = S.lvc[level];
+                if (level + 1 > J.max_cost) {
+                    L.status = ST_NOT_FOUND;
+                } else {
+                    L.level = level + 1;
+                    S.lvs[level + 1] = size;
+                    S.lvc[level + 1] = 0;
+                    J.lvl_start[level + 1] = size;
+                    J.lvl_count[level + 1] = 0;
+                }
+            }
+            __syncwarp();
+            if (level + 1 > J.max_cost) {
+                if (lane == 0) plan.small = 0;
+                return;
+            }
+            level++;
+        }
+        plan_level<kAnyWidth, true>(J, level, S.lvs, S.lvc, S.seg, plan);
+        const uint64_t T = plan.total;
+        const uint64_t limit = umin64(J.cache_alloc, J.cap);
+        const bool fits = T <= kSortMax && T <= J.chunk_max && size + T <= J.small_rows && size + T <= limit &&
+                          !(J.handover && T > J.handover && size > 0);
+        if (fits && T == 0) {  // an empty level: on to the next
+            count = true;
+            continue;
+        }
+        if (fits) tile_setup(S, plan.nseg, 0, T, s_tiles, 32);
+        if (lane == 0) {
+            *s_found = kNone;
+            plan.small = fits && *s_tiles <= solo_tiles &&
+                         !(J.yield_ns && globaltimer_ns() - J.t_start > J.yield_ns);
+        }
+        return;
+    }
+}
+
+// Returns whether the answer is in the level entered last (its index in
+// st->found, its plan in S.seg); else the leader's loop goes on from L.
+template <uint32_t WT>
+__device__ bool small_levels(const SolveJob &J, SolveState *st, Shared &S, const Cta &K, uint32_t solo_tiles) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t W = WT ? WT : J.W;
+    Lead &L = *K.L;
+    Plan &plan = *K.plan;
+    uint32_t *bits = S.solo_bits, *keep = S.solo_pref;
+    const unsigned long long *ent = S.sortbuf;
+    if (wid == 0) small_next(J, S, L, plan, K.tiles, K.found, L.level, L.size, false, solo_tiles);
+    __syncthreads();
+    for (;;) {
+        if (!plan.small) return false;
+        const uint32_t level = L.level, size = L.size, nseg = plan.nseg, C = (uint32_t)plan.total, nw = (C + 31) / 32;
+        const uint32_t ntiles = (uint32_t)*K.tiles;
+        uint32_t s = 0;
+        for (uint32_t t = wid; t < ntiles; t += nwarps) {
+            while (s + 1 < nseg && S.tile_first[s + 1] <= t) s++;
+            small_tile<WT>(J, S, st, S.seg[s], S.tiles[s], t - (uint32_t)S.tile_first[s], K.wm, K.found);
+        }
+        __syncthreads();
+        if (*K.found != kNone) {
+            for (uint32_t w = tid; w < nw; w += blockDim.x) bits[w] = 0;
+            if (tid == 0) st->found = *K.found;
+            __syncthreads();
+            return true;
+        }
+        // the marks whose slot still names them
+        for (uint32_t w = wid; w < nw; w += nwarps) {
+            const uint32_t xl = 32 * w + lane, b = bits[w];
+            bool mine = (b >> lane) & 1u;
+            if (mine) mine = (S.sm_table[(uint32_t)ent[xl] & 0xFFFFu] & 0x1FFFFu) == (kSmPending | xl);
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, mine);
+            if (lane == 0) {
+                keep[w] = m;
+                bits[w] = 0;
+            }
+        }
+        __syncthreads();
+        // survivors before each word (nw <= 64: two words per lane of every warp)
+        const uint32_t k0 = 2 * lane < nw ? keep[2 * lane] : 0u, k1 = 2 * lane + 1 < nw ? keep[2 * lane + 1] : 0u;
+        uint32_t incl = __popc(k0) + __popc(k1);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if (lane >= (uint32_t)d) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31), before = incl - __popc(k0) - __popc(k1);
+        if (wid == 0 && nwarps > 1) {
+            small_next(J, S, L, plan, K.tiles, K.found, level, size + total, true, solo_tiles);
+        } else {
+            // warps 1.. append (warp 0 plans; alone, it appends first)
+            const uint32_t a0 = nwarps > 1 ? wid - 1 : 0u, step = nwarps > 1 ? nwarps - 1 : 1u;
+            for (uint32_t w = a0; w < nw; w += step) {
+                const uint32_t e0 = __shfl_sync(0xFFFFFFFFu, before, w >> 1), p0 = __shfl_sync(0xFFFFFFFFu, k0, w >> 1);
+                const uint32_t m = keep[w], base = e0 + ((w & 1u) ? __popc(p0) : 0u);
+                if (!((m >> lane) & 1u)) continue;
+                const uint32_t xl = 32 * w + lane, k = size + base + __popc(m & ((1u << lane) - 1u));
+                const unsigned long long e = ent[xl];
+                const uint32_t q = (uint32_t)e & 0xFFFFu, l = (uint32_t)(e >> 16) & 0xFFFFu, r = (uint32_t)(e >> 32) & 0xFFFFu;
+                const uint32_t *src = S.sm_tmp + xl * W;
+                uint32_t *ds = S.sm_rows + k * W, *dg = J.cs + (uint64_t)k * W;
+                for (uint32_t b = 0; b < W; b++) {
+                    const uint32_t v = src[b];
+                    ds[b] = v;
+                    dg[b] = v;
+                }
+                J.bp_op[k] = (uint8_t)(e >> 48);
+                J.bp_l[k] = l;
+                J.bp_r[k] = r == 0xFFFFu ? kNoRight : r;
+                S.sm_table[q] = (S.sm_table[q] & 0xFFFE0000u) | k;
+            }
+            if (nwarps == 1) {
+                __syncwarp();
+                small_next(J, S, L, plan, K.tiles, K.found, level, size + total, true, solo_tiles);
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // The leader's search loop (Alg. 1): level after level, chunk after chunk,
 // until the answer, not_found, out-of-memory, or a request for more memory.
 // With allow_team, large chunks are handed to every CTA of the launch.
 // Returns -1 when a grid barrier gave up, else 0; the final state is written
 // back to `st`.
-template <uint32_t WC>
+// SMALL: the launch may start with its languages in shared memory
+template <uint32_t WC, bool SMALL>
 __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const Cta &K, bool allow_team,
                            uint32_t &bar_epoch) {
     const uint32_t tid = threadIdx.x, wid = tid >> 5;
@@ -2548,6 +2879,14 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
     REI_TSPAN_END(st, t_init, 17);
 
     bool found = false;
+    if (SMALL && L.smode && L.status == ST_RUNNING && L.level <= J.max_cost) {
+        // (with a team, a level of more tiles than solo_tiles is the team's)
+        const uint32_t solo = allow_team ? J.solo_tiles : 0xFFFFFFFFu;
+        if (WC == 1 || (WC == kAnyWidth && J.W == 1)) found = small_levels<1>(J, st, S, K, solo);
+        else if (WC == 2 || (WC == kAnyWidth && J.W == 2)) found = small_levels<2>(J, st, S, K, solo);
+        else if (WC == 4 || (WC == kAnyWidth && J.W == 4)) found = small_levels<4>(J, st, S, K, solo);
+        else found = small_levels<0>(J, st, S, K, solo);
+    }
     uint32_t planned = 0xFFFFFFFFu;  // the level whose plan is in S.seg / s_plan
     // end of a level (thread 0): count it, check the cache cap, enter the next one
     auto end_level = [&](uint32_t level, uint32_t nseg) {
@@ -2590,7 +2929,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
     };
     // per-phase wall time of the leader (ns): plan, solo chunk, team chunk, level end
     unsigned long long tm[4] = {0, 0, 0, 0}, tcnt[3] = {0, 0, 0};
-    for (;;) {
+    while (!found) {
         const unsigned long long t_it = globaltimer_ns();
         const uint32_t status = L.status, level = L.level, size = L.size, full = L.full, otf = L.otf;
         const uint64_t pos = L.chunk_pos;
@@ -2791,7 +3130,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
 }
 
 // the search of one problem by its team of CTAs (the first one leads)
-template <uint32_t WC>
+template <uint32_t WC, bool SMALL = true>
 __device__ __forceinline__ void solve_body(const SolveJob &J, uint32_t &bar_epoch) {
     SolveState *st = J.st;
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -2875,7 +3214,7 @@ __device__ __forceinline__ void solve_body(const SolveJob &J, uint32_t &bar_epoc
     }
 
     // ---- CTA 0 leads
-    if (lead_search<WC>(J, st, S, K, true, bar_epoch) < 0) return;
+    if (lead_search<WC, SMALL>(J, st, S, K, true, bar_epoch) < 0) return;
     REI_TSPAN_BEGIN(t_cl);
     const uint32_t status = ld_relaxed_u32(&st->status);
     if (L.cleaned) {

@@ -91,7 +91,7 @@ __device__ uint32_t solve_in_slot(SolveJob &J, const SlotMem &m, uint32_t slot, 
     carve_shared(J, S, smem_raw, &wm);
     const Cta K{s_plan, s_red, s_tiles, s_found, s_marked, L, wm};
     uint32_t epoch = 0;
-    lead_search<kAnyWidth>(J, st, S, K, false, epoch);
+    lead_search<kAnyWidth, false>(J, st, S, K, false, epoch);
     const uint32_t status = st->status;
     if (status == ST_FOUND || status == ST_NOT_FOUND || status == ST_OOM) {
         clean_table(J, L->smode ? 0u : L->size, L->clean_marks, 1, 0);
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256, 2) k_solve_groups(const BatchJob *jobs, c
     }
     __syncthreads();
     uint32_t epoch = 0;
-    solve_body<kAnyWidth>(J, epoch);
+    solve_body<kAnyWidth, false>(J, epoch);
     if (team_rank_of(J) == 0 && threadIdx.x == 0)
         report_slot(J, ld_relaxed_u32(&J.st->status), slot, globaltimer_ns() - s_t0, *bj.out);
 }
