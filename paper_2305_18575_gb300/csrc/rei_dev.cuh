@@ -123,7 +123,7 @@ struct SolveState {
     uint32_t otf;             // OnTheFly mode
     uint32_t partial_level;   // first level not completely cached
     unsigned long long found; // level-local index of the answer, or kNone
-    uint32_t marked;          // the current chunk has marked candidates
+    uint32_t marked;          // the number (ChunkArgs::epoch) of the last chunk with marked candidates
     uint32_t ans_op, ans_l, ans_r, ans_cost;
     uint32_t tree_len;        // postfix tokens written
     uint64_t candidates;      // completed levels

@@ -1906,6 +1906,17 @@ __device__ inline void solo_append(const SolveJob &J, SolveState *st, Shared &S,
 constexpr uint32_t kDynTilesPerWarp = 32;
 constexpr uint32_t kGrab = 4;
 
+// the slot of a marked candidate, checked before it is followed: one outside
+// the table was not written by this chunk (never expected), and the search is
+// stopped with an error instead
+__device__ __forceinline__ uint32_t mark_slot(const SolveJob &J, uint32_t j) {
+    const uint32_t q = ldcg(J.slotpos + j);
+    if (q <= J.table_mask) return q;
+    atomicCAS(&J.st->err, 0u, 7u);
+    atomicExch(&J.st->status, (uint32_t)ST_TIMEOUT);
+    return 0;
+}
+
 // Visit the marked candidates of a chunk of C (whole warps of the team: this
 // one is number gw of nw): f(j, on, drop) gets four candidates a lane at a time
 // (those with on[u]) and says which marks to clear.  A warp takes up to 32
@@ -2079,8 +2090,11 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
                 }
             }
         }
-        // (one word tells every CTA, after the barrier, that the chunk has marks)
-        if (marked) st->marked = 1;
+        // (one word tells every CTA, after the barrier, that the chunk has
+        // marks: the chunk's number, since a chunk without marks ends at that
+        // barrier, and a CTA slow to read the word there may find what the next
+        // chunk's tiles have set already)
+        if (marked) st->marked = a.epoch;
 #ifdef REI_TIMING
         if (lane == 0) atomicMax(&s_wmax, globaltimer_ns() - t_loop0);
         __syncthreads();
@@ -2138,7 +2152,7 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
     REI_TMARK(!full, 1);
     if (*s_found != kNone) return 1;
     // no new language: nothing to append
-    if (!dedup || !*s_marked) return 0;
+    if (!dedup || *s_marked != a.epoch) return 0;
     const uint64_t C = a.ce0 - a.cs0;
 
     // ---- phase B: drop the marks whose slot no longer names them
@@ -2146,7 +2160,7 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
               [&](const uint32_t (&j)[4], const bool (&on)[4], bool (&drop)[4]) {
                   uint32_t q[4], m[4];
 #pragma unroll
-                  for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? ldcg(J.slotpos + j[u]) : 0u;
+                  for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? mark_slot(J, j[u]) : 0u;
                   // (a marked slot is of this chunk: its entry's low half tells)
 #pragma unroll
                   for (uint32_t u = 0; u < 4; u++)
@@ -2282,7 +2296,7 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     const uint32_t i = i0 + u * nt;
-                    if (i < cnt) q[u] = ldcg(J.slotpos + list[i]);
+                    if (i < cnt) q[u] = mark_slot(J, list[i]);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
@@ -2505,7 +2519,7 @@ __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nm
         each_mark(J, nmarks, t >> 5, nt >> 5, [&](const uint32_t (&j)[4], const bool (&on)[4], bool (&drop)[4]) {
             uint32_t q[4];
 #pragma unroll
-            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] && !all ? ldcg(J.slotpos + j[u]) : 0u;
+            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] && !all ? mark_slot(J, j[u]) : 0u;
 #pragma unroll
             for (uint32_t u = 0; u < 4; u++) {
                 drop[u] = on[u];
@@ -3046,7 +3060,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
         }
         if (r == 1) {
             // (a chunk with shared-memory bookkeeping has emptied its slots itself)
-            if (tid == 0 && ld_relaxed_u32(&st->marked)) L.clean_marks = (uint32_t)(a.ce0 - a.cs0);
+            if (tid == 0 && ld_relaxed_u32(&st->marked) == a.epoch) L.clean_marks = (uint32_t)(a.ce0 - a.cs0);
             found = true;
             break;
         }
