@@ -78,6 +78,7 @@ struct rei_ctx {
     int64_t opt_chunk = 0, opt_grid = 0, opt_keep = 0, opt_cache_init = 0, opt_solo_tiles = -1, opt_small_rows = -1;
     int64_t opt_fused = 1, opt_exact = 1;
     uint64_t opt_handover = 1ull << 22;  // levels of more candidates leave the fused launch
+    uint32_t share = 1;                  // this context's relaunches take one in `share` of the GPU's SMs
     uint64_t opt_yield_us = 500;         // batched / served problems longer than this continue on the whole GPU
     bool phases = getenv("REI_PHASES") != nullptr;  // per-solve timing report on stderr (diagnostics)
     unsigned long long fused_launch_id = 0;         // ids of this context's fused launches (only grow)
@@ -524,7 +525,7 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     int bps = 0;
     CK(solve_fused_occupancy(threads, smem, &bps));
     if (bps < 1) return REI_EBUSY;
-    uint32_t grid = std::min<uint32_t>((uint32_t)(c->sm_count * bps), kMaxTeam);
+    uint32_t grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
     if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
     if ((s = ensure(c, c->blk, 4ull * grid))) return s;
     if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
@@ -823,7 +824,10 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     int bps = 0;
     CK(solve_occupancy(W, threads, smem, &bps));
     if (bps < 1) return REI_ECUDA;
-    grid = std::min<uint32_t>((uint32_t)(c->sm_count * bps), kMaxTeam);
+    // (a helper's launch takes its share of the SMs, whatever CTAs of this
+    // width fit one: launches side by side whose CTAs wait for each other must
+    // fit the GPU together)
+    grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
     if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
 
     // a chunk costs a fixed ~15 us of barriers and bookkeeping, so the
@@ -1787,8 +1791,8 @@ rei_status run_batch(rei_ctx *c, const rei_problem *probs, const std::vector<uin
             h->opt_fused = c->opt_fused;
             h->opt_exact = c->opt_exact;
             h->opt_handover = c->opt_handover;
-            const int64_t share = std::max<int64_t>(1, (int64_t)c->sm_count * 2 / nuse);  // (k_solve: 2 CTAs per SM)
-            h->opt_grid = c->opt_grid > 0 ? std::min<int64_t>(c->opt_grid, share) : share;
+            h->share = nuse;
+            h->opt_grid = c->opt_grid;
             l0[k] = h->launches;
             th.emplace_back([&, h] {
                 cudaSetDevice(h->device);
