@@ -291,6 +291,7 @@ struct GroupArgs {
     // candidates, tmp_words words of candidate rows; the bitmaps start zeroed
     uint32_t *tmp, *pending, *slotpos, *bitmap;
     uint64_t chunk, tmp_words;
+    uint64_t yield_ns;               // a search still running after this long parks again (0 = never)
 };
 
 struct BatchArgs {

@@ -168,11 +168,12 @@ __global__ void __launch_bounds__(256, 2) k_solve_groups(const BatchJob *jobs, c
         J.chunk_max = umin64(umin64(G.chunk, G.tmp_words / J.W), (J.table_mask + 1) / 2 - J.cache_alloc);
         J.team_base = g * G.group_ctas;
         J.team_size = G.group_ctas;
-        J.yield_ns = 0;
+        J.yield_ns = G.yield_ns;
         J.solo_tiles = 64;
         J.small_rows = 0;
         J.handover = 0;
         s_t0 = globaltimer_ns();
+        J.t_start = s_t0;
         // (the leader continues the parked search; the other CTAs read no
         // state before its first command)
         if (team_rank_of(J) == 0) {
