@@ -215,6 +215,12 @@ constexpr uint32_t kAnyWidth = 0, kWide = 8, kWidest = 20;
 
 constexpr uint32_t kSortMax = 2048;  // candidates of a chunk CTA 0 runs with shared-memory bookkeeping
 
+// The shared-memory start: languages of up to kSmallMaxW words, chunks of up to
+// small_tmp(W) candidates (wider languages fill the memory with fewer: their
+// first levels, of tens to hundreds of candidates, still fit)
+constexpr uint32_t kSmallMaxW = 16;
+__host__ __device__ inline uint32_t small_tmp(uint32_t W) { return W <= 8 ? kSortMax : 512u; }
+
 // Candidates per tile of a concatenation or union segment: 32 (one per lane),
 // or 32 * reg_per (reg_per per lane, built side by side in registers) for
 // 1-word languages and, in the relaunch of 2-word ones, for chunks of kRegChunk
@@ -248,16 +254,24 @@ struct Shared {
     // the search's start, while every language fits in CTA 0's shared memory
     uint32_t *sm_rows;       // small_rows rows of W words: the cached languages
     uint32_t *sm_table;      // 2 * small_rows slots: fp (15 bits) | pending | row or candidate
-    uint32_t *sm_tmp;        // kSortMax rows: the candidates of the current chunk
+    uint32_t *sm_tmp;        // small_tmp rows: the candidates of the current chunk
+    uint32_t *sm_bp;         // the cached languages' back-pointers (bp_pack), kept for the answer
     uint32_t *lvs, *lvc;     // level table (start, count per cost), mirrored in shared memory
     uint32_t *warp_mem;      // per warp: lw[W], A[32*Ws], B[32*Ws]
     uint32_t warp_words;
 };
 
+// a language of the shared-memory start: operator, left and right operand in one
+// word (rows are below 2^14; a leaf's left is its symbol; no right: zero)
+__device__ __forceinline__ uint32_t bp_pack(uint32_t op, uint32_t l, uint32_t r) {
+    return op << 28 | (r & 0x3FFFu) << 14 | l;
+}
+
 // the search state CTA 0 keeps in shared memory while it leads; written back
 // to the global SolveState when the launch ends
 struct Lead {
     uint32_t status, level, size, full, otf, partial_level;
+    uint32_t sm_size;  // languages whose back-pointers are in shared memory
     uint32_t smode;  // languages and their uniqueness table live in shared memory
     // the answer was found and the other CTAs were told to empty the table
     // (rows and marked candidates given) while the leader writes out the answer
@@ -1473,7 +1487,23 @@ __device__ inline uint32_t emit_tree(const SolveJob &J, uint32_t op, uint32_t l,
 // (in every lane), or falls back to emit_tree when the tree does not fit.
 constexpr uint32_t kTreeNodes = 480;  // nodes the scratch holds (7 arrays + depth starts)
 constexpr uint32_t kTreeScratchWords = 7 * kTreeNodes + kTreeNodes + 1;
-__device__ inline uint32_t emit_tree_warp(const SolveJob &J, uint32_t op, uint32_t l, uint32_t r, uint32_t *scr) {
+// The languages below sm_size have their back-pointers in shared memory (sm_bp):
+// an answer's subtrees are mostly of the first levels, and a depth whose nodes
+// all are costs no round trip to the L2.
+__device__ inline uint32_t emit_tree_warp(const SolveJob &J, uint32_t op, uint32_t l, uint32_t r, uint32_t *scr,
+                                          const uint32_t *sm_bp, uint32_t sm_size) {
+    auto back = [&](uint32_t e, uint32_t &o, uint32_t &a, uint32_t &b) {
+        if (e < sm_size) {
+            const uint32_t w = sm_bp[e];
+            o = w >> 28;
+            a = w & 0x3FFFu;
+            b = (w >> 14) & 0x3FFFu;
+        } else {
+            o = *(volatile const uint8_t *)(J.bp_op + e);
+            a = ldcg(J.bp_l + e);
+            b = ldcg(J.bp_r + e);
+        }
+    };
     const uint32_t lane = threadIdx.x & 31;
     uint32_t *nop = scr, *na = nop + kTreeNodes, *nb = na + kTreeNodes, *c0 = nb + kTreeNodes;
     uint32_t *c1 = c0 + kTreeNodes, *sz = c1 + kTreeNodes, *pos = sz + kTreeNodes, *dep = pos + kTreeNodes;
@@ -1511,14 +1541,9 @@ __device__ inline uint32_t emit_tree_warp(const SolveJob &J, uint32_t op, uint32
             }
             if (k) {
                 const uint32_t e0 = na[v];
-                uint32_t op0 = *(volatile const uint8_t *)(J.bp_op + e0), l0 = ldcg(J.bp_l + e0), r0 = ldcg(J.bp_r + e0);
-                uint32_t op1 = 0, l1 = 0, r1 = 0;
-                if (k == 2) {
-                    const uint32_t e1 = nb[v];
-                    op1 = *(volatile const uint8_t *)(J.bp_op + e1);
-                    l1 = ldcg(J.bp_l + e1);
-                    r1 = ldcg(J.bp_r + e1);
-                }
+                uint32_t op0, l0, r0, op1 = 0, l1 = 0, r1 = 0;
+                back(e0, op0, l0, r0);
+                if (k == 2) back(nb[v], op1, l1, r1);
                 nop[at] = op0;
                 na[at] = l0;
                 nb[at] = r0;
@@ -1630,7 +1655,7 @@ __host__ __device__ inline size_t search_smem_bytes(uint32_t W, uint32_t n, uint
     size_t b = sizeof(Seg) * seg_cap + sizeof(uint64_t) * (seg_cap + 1) + sizeof(SegTile) * seg_cap;
     b += sizeof(unsigned long long) * kSortMax;
     b += sizeof(uint32_t) * (2 * (kSortMax / 32) + 4);
-    if (small_rows) b += sizeof(uint32_t) * ((size_t)small_rows * W + 2 * small_rows + (size_t)kSortMax * W);
+    if (small_rows) b += sizeof(uint32_t) * ((size_t)small_rows * (W + 3) + (size_t)small_tmp(W) * W);
     b += 2 * sizeof(uint32_t) * seg_cap;
     b += 2 * sizeof(uint32_t) * W;
     if (gt_in_smem) b += sizeof(uint32_t) * (((n + 1 + G + max_len + 2) + 3) & ~3u);
@@ -1765,6 +1790,7 @@ __device__ inline void smem_append(const SolveJob &J, Shared &S, const ChunkArgs
         J.bp_op[k] = (uint8_t)op;
         J.bp_l[k] = l;
         J.bp_r[k] = r;
+        S.sm_bp[k] = bp_pack(op, l, r);
         S.sm_table[q] = (S.sm_table[q] & 0xFFFE0000u) | k;
     }
     __syncthreads();
@@ -1800,7 +1826,10 @@ __device__ inline void switch_to_global(const SolveJob &J, Shared &S, Lead *L) {
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) L->smode = 0;
+    if (threadIdx.x == 0) {
+        L->smode = 0;
+        L->sm_size = rows;
+    }
     __syncthreads();
     REI_TSPAN_END(J.st, t_sw, 16);
 }
@@ -2412,14 +2441,16 @@ __device__ inline void carve_shared(const SolveJob &J, Shared &S, uint8_t *smem_
     p += sizeof(uint32_t) * (kSortMax / 32);
     S.solo_pref = reinterpret_cast<uint32_t *>(p);
     p += sizeof(uint32_t) * (kSortMax / 32 + 4);
-    S.sm_rows = S.sm_table = S.sm_tmp = nullptr;
+    S.sm_rows = S.sm_table = S.sm_tmp = S.sm_bp = nullptr;
     if (J.small_rows) {
         S.sm_rows = reinterpret_cast<uint32_t *>(p);
         p += sizeof(uint32_t) * J.small_rows * W;
         S.sm_table = reinterpret_cast<uint32_t *>(p);
         p += sizeof(uint32_t) * 2 * J.small_rows;
         S.sm_tmp = reinterpret_cast<uint32_t *>(p);
-        p += sizeof(uint32_t) * kSortMax * W;
+        p += sizeof(uint32_t) * small_tmp(W) * W;
+        S.sm_bp = reinterpret_cast<uint32_t *>(p);
+        p += sizeof(uint32_t) * J.small_rows;
     }
     for (uint32_t i = tid; i < kSortMax / 32; i += blockDim.x) S.solo_bits[i] = 0;
     S.lvs = reinterpret_cast<uint32_t *>(p);
@@ -2744,7 +2775,7 @@ __device__ inline void small_next(const SolveJob &J, Shared &S, Lead &L, Plan &p
         plan_level<kAnyWidth, true>(J, level, S.lvs, S.lvc, S.seg, plan);
         const uint64_t T = plan.total;
         const uint64_t limit = umin64(J.cache_alloc, J.cap);
-        const bool fits = T <= kSortMax && T <= J.chunk_max && size + T <= J.small_rows && size + T <= limit &&
+        const bool fits = T <= small_tmp(J.W) && T <= J.chunk_max && size + T <= J.small_rows && size + T <= limit &&
                           !(J.handover && T > J.handover && size > 0);
         if (fits && T == 0) {  // an empty level: on to the next
             count = true;
@@ -2831,6 +2862,7 @@ __device__ bool small_levels(const SolveJob &J, SolveState *st, Shared &S, const
                 J.bp_op[k] = (uint8_t)(e >> 48);
                 J.bp_l[k] = l;
                 J.bp_r[k] = r == 0xFFFFu ? kNoRight : r;
+                S.sm_bp[k] = bp_pack((uint32_t)(e >> 48), l, r);
                 S.sm_table[q] = (S.sm_table[q] & 0xFFFE0000u) | k;
             }
             if (nwarps == 1) {
@@ -2859,6 +2891,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
         L.cleaned = 0;
         L.clean_marks = 0;
         L.epoch = 0;
+        L.sm_size = 0;
         L.status = st->status;
         L.level = st->level;
         L.size = st->size;
@@ -3029,7 +3062,7 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
         REI_TSPAN_END(st, t_ts, 19);
         const bool team = allow_team && *K.tiles > (uint64_t)J.solo_tiles;
         // the shared-memory start ends before a chunk it cannot hold
-        if (L.smode && (team || !dedup || C > kSortMax || (uint64_t)size + C > J.small_rows))
+        if (L.smode && (team || !dedup || C > small_tmp(J.W) || (uint64_t)size + C > J.small_rows))
             switch_to_global(J, S, &L);
         const unsigned long long t_chunk = globaltimer_ns();
         if (tid == 0) tm[0] += t_chunk - t_it;
@@ -3116,7 +3149,8 @@ __device__ int lead_search(const SolveJob &J, SolveState *st, Shared &S, const C
             l = __shfl_sync(0xFFFFFFFFu, l, 0);
             r = __shfl_sync(0xFFFFFFFFu, r, 0);
             // (the chunk's shared scratch is free once its answer is known)
-            const uint32_t nt = emit_tree_warp(J, op, l, r, reinterpret_cast<uint32_t *>(S.sortbuf));
+            const uint32_t nt = emit_tree_warp(J, op, l, r, reinterpret_cast<uint32_t *>(S.sortbuf), S.sm_bp,
+                                               L.smode ? L.size : L.sm_size);
             if (lane == 0) {
                 st->tree_len = nt;
                 L.status = ST_FOUND;

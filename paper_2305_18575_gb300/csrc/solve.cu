@@ -47,6 +47,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_solve_fused(const __grid_c
             unsigned long long *si = reinterpret_cast<unsigned long long *>(F.sj.info);
             for (uint32_t i = threadIdx.x; i < sizeof(StageInfo) / 8; i += blockDim.x) si[i] = 0;
         }
+        // (CTA 0 keeps the job in shared memory)
+        {
+            const unsigned long long *src = reinterpret_cast<const unsigned long long *>(&F.tmpl);
+            unsigned long long *dst = reinterpret_cast<unsigned long long *>(&J);
+            for (uint32_t i = threadIdx.x; i < sizeof(SolveJob) / 8; i += blockDim.x) dst[i] = src[i];
+        }
         for (uint32_t c = threadIdx.x; c < F.tmpl.max_cost + 2; c += blockDim.x) {
             F.tmpl.lvl_start[c] = 0;
             F.tmpl.lvl_count[c] = 0;
@@ -69,8 +75,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_solve_fused(const __grid_c
         }
         __syncthreads();
         if (threadIdx.x == 0) {
+            // (completed in place: copying the job through one thread's
+            // registers took 3 us of every solve)
             const StageInfo I = *F.sj.info;
-            SolveJob j = F.tmpl;
+            SolveJob &j = J;
             bool ok = I.status == SE_OK;
             if (ok) {
                 j.n = I.n;
@@ -98,7 +106,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_solve_fused(const __grid_c
                 const uint32_t warps = blockDim.x / 32;
                 j.gt_in_smem = search_smem_bytes(W, I.n, I.G, I.max_len, j.seg_cap, true, warps, 0) <= F.smem_cap;
                 j.small_rows = 0;
-                if (F.small_opt && W <= 8) {
+                if (F.small_opt && W <= kSmallMaxW) {
                     uint32_t r = F.small_opt != 0xFFFFFFFFu ? F.small_opt : W <= 2 ? 4096u : W <= 4 ? 2048u : 1024u;
                     for (; r >= 256; r >>= 1)
                         if (search_smem_bytes(W, I.n, I.G, I.max_len, j.seg_cap, j.gt_in_smem, warps, r) <= F.smem_cap)
@@ -109,7 +117,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_solve_fused(const __grid_c
                      search_smem_bytes(W, I.n, I.G, I.max_len, j.seg_cap, j.gt_in_smem, warps, j.small_rows) <=
                          F.smem_cap;
             }
-            J = j;  // (CTA 0 keeps the job in shared memory)
             if (!ok) st->status = ST_RESTAGE;
             s_go = ok ? 1u : 0u;
         }
