@@ -208,8 +208,8 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     NA_CK(cudaGetDevice(&device));
     unsigned char *scratch = nullptr;
     NA_CK(scratch_address(device, &scratch));
-    cudaDeviceProp prop;
-    NA_CK(cudaGetDeviceProperties(&prop, device));
+    int sm_count = 0;
+    NA_CK(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device));
 
     Carve cv{scratch, 0, (size_t)REI_NOALLOC_SCRATCH_BYTES};
     uint8_t *d_bytes = (uint8_t *)cv.take(kInputBytes);
@@ -305,7 +305,7 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     NA_CK(solve_smem_max(W, &smem_max));
     const uint32_t seg_cap = 2 * max_cost + 4;
     bool gt_smem = 4ull * (n + 1 + G + max_len + 2) <= 96 * 1024;
-    uint32_t warps = 8;
+    uint32_t warps = 16;
     size_t smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps);
     while (smem > smem_max && warps > 1) {
         warps /= 2;
@@ -313,7 +313,7 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     }
     if (smem > smem_max && gt_smem) {
         gt_smem = false;
-        warps = 8;
+        warps = 16;
         smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps);
         while (smem > smem_max && warps > 1) {
             warps /= 2;
@@ -321,10 +321,22 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
         }
     }
     if (smem > smem_max) NA_RET(REI_EINVAL);
+    // the first levels in CTA 0's shared memory, as the plain solve's first
+    // launch has them (with 8-warp CTAs, no shared-memory start and every CTA
+    // planning each level, four medium searches took 625 us, so 520 us)
+    uint32_t small_rows = 0;
+    if (W <= 8) {
+        uint32_t r = W <= 2 ? 4096u : W <= 4 ? 2048u : 1024u;
+        while (r >= 256 && solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps, r) > smem_max) r >>= 1;
+        if (r >= 256) {
+            small_rows = r;
+            smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps, r);
+        }
+    }
     int bps = 0;
     NA_CK(solve_occupancy(W, 32 * warps, smem, &bps));
     if (bps < 1) NA_RET(REI_ECUDA);
-    const uint32_t grid = std::min<uint32_t>(kMaxTeam, (uint32_t)(prop.multiProcessorCount * bps));
+    const uint32_t grid = std::min<uint32_t>(kMaxTeam, (uint32_t)(sm_count * bps));
 
     // what must start cleared: table, survivor bitmap, level sizes
     NA_CK(cudaMemsetAsync(d_table, 0xFF, 8ull * tslots, stream));
@@ -392,7 +404,11 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     j.tstack = d_tstack;
     j.trace = d_trace;
     j.gt_in_smem = gt_smem ? 1 : 0;
-    j.solo_tiles = 8 * warps;
+    j.solo_tiles = 64;
+    j.small_rows = small_rows;
+    // (what the array has left holds the chunk plans CTA 0 publishes; without
+    // room for them every CTA plans)
+    j.plan = (uint64_t *)cv.take(8 * plan_words(seg_cap));
     NA_CK(launch_solve(&j, grid, 32 * warps, smem, stream));
     struct {
         SolveState s;
