@@ -801,11 +801,37 @@ __device__ __forceinline__ bool mark_tile(const SolveJob &J, uint32_t xl, uint32
     return true;
 }
 
+// A tile's 32 operand rows (nrow of them there, zero beyond), which lie one after
+// another at src, into A (row stride Ws), with f applied to every word.  U loads
+// a lane are in flight before any is stored: one after another (U = 1) a tile of
+// 32-word languages takes 32 round trips to the L2 for its operands.  U = 8 for
+// the widest languages (|ic| near 1000 to cost 12: 8.1 -> 7.0 ms), 4 for 4 to 16
+// words at 64 registers (|ic| 65-128: 4.6 -> 4.4 ms; 8 spilled and cost 12-word
+// searches 4 %), 1 in the first launch, whose tiles are small.
+template <uint32_t WT, uint32_t U, class F>
+__device__ __forceinline__ void load_rows(uint32_t *A, const uint32_t *src, uint32_t Wr, uint32_t Ws, uint32_t nrow, F f) {
+    const uint32_t lane = threadIdx.x & 31, W = WT ? WT : Wr;
+    const uint32_t wlog = (W & (W - 1)) == 0 ? (uint32_t)(__ffs(W) - 1) : 32u;
+    const uint32_t have = nrow * W;
+    for (uint32_t i0 = lane; i0 < 32 * W; i0 += 32 * U) {
+        uint32_t v[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; u++) v[u] = i0 + 32 * u < have ? ldop(src + i0 + 32 * u) : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < U; u++) {
+            const uint32_t i = i0 + 32 * u;
+            if (i >= 32 * W) continue;
+            const uint32_t j = wlog < 32 ? i >> wlog : i / W, b = i - j * W;
+            A[j * Ws + b] = i < have ? f(v[u], b) : 0u;
+        }
+    }
+}
+
 // build the CSs of one tile into A (candidate-major, row stride Ws), then test
 // precision and insert; lanes with !valid only help with the warp collectives.
 // WT > 0 fixes the language width at compile time (W = WT), 0 reads it from T.
 // Returns whether any candidate was marked in the chunk's bitmap.
-template <uint32_t WT>
+template <uint32_t WT, uint32_t U = 1>
 __device__ bool run_tile(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile, uint32_t *wm) {
     const SolveJob &J = *T.J;
     const Shared &S = *T.S;
@@ -871,10 +897,7 @@ __device__ bool run_tile(const TileCtx &T, const Seg &sg, const SegTile &tl, uin
         __syncwarp();
     } else if (sg.op == OP_OPT) {
         const uint32_t *src = cs + (uint64_t)(sg.lbase + first) * W;
-        for (uint32_t i = lane; i < 32 * W; i += 32) {
-            TILE_JB(i, j, b);
-            A[j * Ws + b] = j < nrow ? ldop(src + i) : 0u;
-        }
+        load_rows<WT, U>(A, src, W, Ws, nrow, [](uint32_t v, uint32_t) { return v; });
         __syncwarp();
         A[lane * Ws] |= 1u;  // eps is ic word 0
         __syncwarp();
@@ -883,20 +906,14 @@ __device__ bool run_tile(const TileCtx &T, const Seg &sg, const SegTile &tl, uin
         const uint32_t *src = cs + (uint64_t)(sg.rbase + first) * W;
         for (uint32_t b = lane; b < W; b += 32) lw[b] = ldop(l + b);
         __syncwarp();
-        for (uint32_t i = lane; i < 32 * W; i += 32) {
-            TILE_JB(i, j, b);
-            A[j * Ws + b] = j < nrow ? (lw[b] | ldop(src + i)) : 0u;
-        }
+        load_rows<WT, U>(A, src, W, Ws, nrow, [&](uint32_t v, uint32_t b) { return lw[b] | v; });
         __syncwarp();
     } else {
         // CAT / STAR: bit-sliced over 32 operands (the right ones of a
         // concatenation, its left ones when swapped, or a star's only ones)
         const uint32_t base = sg.op == OP_STAR ? sg.lbase : swapped ? sg.lbase : sg.rbase;
         const uint32_t *src = cs + (uint64_t)(base + first) * W;
-        for (uint32_t i = lane; i < 32 * W; i += 32) {
-            TILE_JB(i, j, b);
-            A[j * Ws + b] = j < nrow ? ldop(src + i) : 0u;
-        }
+        load_rows<WT, U>(A, src, W, Ws, nrow, [](uint32_t v, uint32_t) { return v; });
         if (sg.op == OP_CAT) {
             // the one operand shared by the tile
             const uint32_t *o = cs + (uint64_t)(swapped ? sg.rbase + col : sg.lbase + row) * W;
@@ -2016,7 +2033,9 @@ __device__ __forceinline__ bool run_tile_of(const TileCtx &T, const Seg &sg, con
         if (WC == 2 && T.reg && (sg.op == OP_CAT || sg.op == OP_ALT)) return run_tile_w2<reg_per<WC>()>(T, sg, tl, tile, wm);
         return run_tile<2>(T, sg, tl, tile, wm);
     }
-    if (WC == 4) return run_tile<4>(T, sg, tl, tile, wm);
+    if (WC == 4) return run_tile<4, 4>(T, sg, tl, tile, wm);
+    if (WC == kWide) return run_tile<0, 4>(T, sg, tl, tile, wm);
+    if (WC == kWidest) return run_tile<0, 8>(T, sg, tl, tile, wm);
     return run_tile<0>(T, sg, tl, tile, wm);
 }
 
