@@ -228,7 +228,7 @@ __host__ __device__ inline uint32_t small_tmp(uint32_t W) { return W <= 8 ? kSor
 // the better one: it spreads a chunk over more warps, and a chunk of a few
 // tiles a warp ends with its slowest tile (in the first launch tiles of 128
 // made medium searches 3 % slower).  The relaunch takes eight 1-word
-// candidates a lane (a deep search 97 ms, with four 100 ms) and four 2-word ones
+// candidates a lane (a deep search 81 ms, with four 86 ms) and four 2-word ones
 // (|ic| 36-42 to cost 20: 9.5 ms; two 9.6 ms, six 10.3 ms, eight 11.3 ms).
 constexpr uint32_t kRegChunk = 64;
 template <uint32_t WC>
@@ -1952,15 +1952,21 @@ __device__ inline void solo_append(const SolveJob &J, SolveState *st, Shared &S,
 constexpr uint32_t kDynTilesPerWarp = 32;
 constexpr uint32_t kGrab = 4;
 
-// the slot of a marked candidate, checked before it is followed: one outside
-// the table was not written by this chunk (never expected), and the search is
-// stopped with an error instead
-__device__ __forceinline__ uint32_t mark_slot(const SolveJob &J, uint32_t j) {
-    const uint32_t q = ldcg(J.slotpos + j);
-    if (q <= J.table_mask) return q;
-    atomicCAS(&J.st->err, 0u, 7u);
-    atomicExch(&J.st->status, (uint32_t)ST_TIMEOUT);
-    return 0;
+// The slots of four marked candidates, checked before they are followed: one
+// outside the table was not written by this chunk (never expected), and the
+// search is stopped with an error instead.  All four are loaded before any is
+// checked, so that their loads overlap.
+__device__ __forceinline__ void check_slots(const SolveJob &J, uint32_t (&q)[4]) {
+    bool bad = false;
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++) {
+        bad |= q[u] > J.table_mask;
+        q[u] = q[u] > J.table_mask ? 0u : q[u];
+    }
+    if (bad) {
+        atomicCAS(&J.st->err, 0u, 7u);
+        atomicExch(&J.st->status, (uint32_t)ST_TIMEOUT);
+    }
 }
 
 // Visit the marked candidates of a chunk of C (whole warps of the team: this
@@ -2208,7 +2214,8 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
               [&](const uint32_t (&j)[4], const bool (&on)[4], bool (&drop)[4]) {
                   uint32_t q[4], m[4];
 #pragma unroll
-                  for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? mark_slot(J, j[u]) : 0u;
+                  for (uint32_t u = 0; u < 4; u++) q[u] = on[u] ? ldcg(J.slotpos + j[u]) : 0u;
+                  check_slots(J, q);
                   // (a marked slot is of this chunk: its entry's low half tells)
 #pragma unroll
                   for (uint32_t u = 0; u < 4; u++)
@@ -2344,8 +2351,9 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     const uint32_t i = i0 + u * nt;
-                    if (i < cnt) q[u] = mark_slot(J, list[i]);
+                    q[u] = i < cnt ? ldcg(J.slotpos + list[i]) : 0u;
                 }
+                check_slots(J, q);
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
                     const uint32_t i = i0 + u * nt;
@@ -2530,15 +2538,18 @@ struct Cta {
 // without clearing it: the slot of every cached row, and the slots of the
 // marked candidates (the first nmarks of a chunk may hold marks) of a chunk
 // that ended with the answer before its survivors were appended; their marks
-// are cleared too.  When the rows are a sixteenth of the slots or more the whole
-// table is written instead, in order: at random addresses the HBM takes 23 G
-// slots a second, in order about 400 G (a search of 35 million 2-word languages
-// took 1.0 ms to empty its table).
+// are cleared too.  When that is the quicker way the whole table is written
+// instead, in order: beyond the L2 (256 MiB and more) the HBM takes 23 G slots a
+// second at random addresses and about 400 G in order, so from a sixteenth of
+// the slots on (a search of 35 million 2-word languages took 1.0 ms to empty its
+// table, 0.27 ms so); within it random addresses run at about 200 G a second,
+// and a table is never full enough.
 __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nmarks, uint32_t team_n,
                                    uint32_t team_r) {
     const uint64_t t = (uint64_t)team_r * blockDim.x + threadIdx.x, nt = (uint64_t)team_n * blockDim.x;
     // (few CTAs are bound by the stores they issue, one a row)
-    const bool all = team_n >= 64 && 16ull * rows > J.table_mask;
+    const uint64_t bytes = (J.table_mask + 1) * (J.exact && !J.direct ? 16 : 8);
+    const bool all = team_n >= 64 && (bytes >= 1ull << 28 ? 16ull : 1ull) * rows > J.table_mask;
     if (all) {
         // (a table is at least 1024 slots from its allocation's start on)
         ulonglong2 *w = reinterpret_cast<ulonglong2 *>(J.table);
@@ -2569,7 +2580,8 @@ __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nm
         each_mark(J, nmarks, t >> 5, nt >> 5, [&](const uint32_t (&j)[4], const bool (&on)[4], bool (&drop)[4]) {
             uint32_t q[4];
 #pragma unroll
-            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] && !all ? mark_slot(J, j[u]) : 0u;
+            for (uint32_t u = 0; u < 4; u++) q[u] = on[u] && !all ? ldcg(J.slotpos + j[u]) : 0u;
+            check_slots(J, q);
 #pragma unroll
             for (uint32_t u = 0; u < 4; u++) {
                 drop[u] = on[u];
