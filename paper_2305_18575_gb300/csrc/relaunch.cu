@@ -8,11 +8,10 @@ namespace rei {
 
 // Two CTAs of 16 warps an SM at 64 registers.  One of 128 registers for 2-word
 // languages, whose tiles keep four candidates a lane with their table slots in
-// registers (|ic| 36-42 to cost 20: 11.7 ms with two CTAs, which spill, 9.5 ms
-// with one; 1-word languages, bound by the L2, lost a tenth with one, 4-word
-// ones a sixth), and from 20 words on, where the warps' tiles leave room for
-// one CTA an SM anyway (32 words to cost 12: 9.1 -> 8.0 ms; 12 words lost a
-// fifth).
+// registers (|ic| 36-42 to cost 20: 9.2 ms, with two CTAs, which spill into the
+// L1, 9.4 ms; 1-word languages, bound by the L2, lost a tenth with one, 4-word
+// ones a sixth), and from 20 words on, where the warps' tiles leave room for one
+// CTA an SM anyway (32 words to cost 12: 9.1 -> 8.0 ms; 12 words lost a fifth).
 template <uint32_t WC>
 __global__ void __launch_bounds__(kSolveThreads, WC == kWidest || WC == 2 ? 1 : 2) k_solve(const __grid_constant__ SolveJob J) {
     uint32_t bar_epoch = 0;

@@ -2091,11 +2091,14 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
         // to warp t mod (warps of the team).
         const bool dyn = full && ntiles >= kDynTilesPerWarp * nw;
         // (1-word languages: longer runs of tiles that share an operand, whose
-        // lookup tables are then built once per run)
-        // Towards the chunk's end the grabs shrink, so that the last warp is a
-        // tile or two behind the others.
-        const uint32_t most = a.bw > 32 ? 4 * kGrab : kGrab;
-        auto grab_at = [&](uint32_t at) { return max(2u, min(most, (ntiles - at) / nw)); };
+        // lookup tables are then built once per run; short runs keep the warps'
+        // operand rows near each other.  1 word: 79 ms a deep search with 8
+        // tiles, 81 with 16, 88 with 32; 2 words: 8.7 ms with 4, 8.8 with 8, 9.2
+        // with 16, 10.2 with 32; 4 words: 3.7 ms with 4, 3.8 with 8.)  Towards
+        // the chunk's end the grabs shrink, so that the last warp is a tile or
+        // two behind the others.
+        const uint32_t most = W == 1 ? 2 * kGrab : kGrab;
+        auto grab_at = [&](uint32_t at) { return max(1u, min(most, (ntiles - at) / nw)); };
         uint32_t t = gw, end = ntiles, step = nw;
         uint32_t nxt = 0, grab = most;
 #ifdef REI_TIMING
