@@ -1396,7 +1396,7 @@ rei_status run_batch(rei_ctx *c, const rei_problem *probs, const std::vector<uin
     if ((s = ensure(c, c->b_tree, tree_bytes * nb))) return s;
     if ((s = ensure(c, c->b_queue, 16))) return s;
     const size_t host_bytes = std::max(P.in_bytes, std::max(sizeof(StageJob), sizeof(BatchJob)) * nb) +
-                              (sizeof(StageInfo) + sizeof(BatchOut) + tree_bytes + 8) * nb + 4096;
+                              (sizeof(StageInfo) + sizeof(BatchOut) + tree_bytes + 16) * nb + 4096;
     if ((s = ensure_pinned(c, host_bytes))) return s;
     CK(cudaStreamSynchronize(c->stream));
     uint8_t *hp = c->h_pin;
@@ -1694,7 +1694,7 @@ rei_status run_batch(rei_ctx *c, const rei_problem *probs, const std::vector<uin
         if (ng > 0) {
             const uint32_t gctas = std::min<uint32_t>(cap / ng, kMaxTeam);
             const uint64_t pstride = plan_words(seg_cap_g);
-            if ((s = ensure(c, c->g_idx, 8ull * ng))) return s;
+            if ((s = ensure(c, c->g_idx, 16ull * ng))) return s;
             if ((s = ensure(c, c->g_blk, 4ull * ng * gctas))) return s;
             if ((s = ensure(c, c->g_plan, 8ull * ng * pstride))) return s;
             // chunks of up to 2^18 candidates (the slot tables' room), rows of
@@ -1712,11 +1712,13 @@ rei_status run_batch(rei_ctx *c, const rei_problem *probs, const std::vector<uin
                 gidx[g] = grp[g].k;
                 gidx[ng + g] = grp[g].slot;
             }
-            CK(cudaMemcpyAsync(c->g_idx.p, gidx, 8ull * ng, cudaMemcpyHostToDevice, c->stream));
+            memset(gidx + 2 * ng, 0, 8ull * ng);  // (the groups' release words)
+            CK(cudaMemcpyAsync(c->g_idx.p, gidx, 16ull * ng, cudaMemcpyHostToDevice, c->stream));
             GroupArgs G{};
             G.slot = A.slot;
             G.prob = (const uint32_t *)c->g_idx.p;
             G.slot_of = (const uint32_t *)c->g_idx.p + ng;
+            G.release = (unsigned long long *)c->g_idx.p + ng;
             G.groups = ng;
             G.group_ctas = gctas;
             G.blk = (uint32_t *)c->g_blk.p;
@@ -2181,19 +2183,21 @@ void continue_in_slots(rei_server *S, std::vector<rei_server::Req> &alone) {
     uint64_t chunk_g = 1ull << 18;
     while (chunk_g > 4096 && chunk_g * wmax_g * ng > (1ull << 28)) chunk_g >>= 1;
     const uint64_t tmp_g = chunk_g * wmax_g, bmw_g = (chunk_g + 31) / 32;
-    if (ensure(c, c->g_idx, 8ull * ng) || ensure(c, c->g_blk, 4ull * ng * gctas) ||
+    if (ensure(c, c->g_idx, 16ull * ng) || ensure(c, c->g_blk, 4ull * ng * gctas) ||
         ensure(c, c->g_plan, 8ull * ng * pstride) || ensure(c, c->g_tmp, 4ull * ng * tmp_g) ||
         ensure(c, c->g_pend, 4ull * ng * chunk_g) || ensure(c, c->g_slotpos, 4ull * ng * chunk_g) ||
-        ensure(c, c->g_bitmap, 4ull * ng * bmw_g) || ensure_pinned(c, 8ull * ng))
+        ensure(c, c->g_bitmap, 4ull * ng * bmw_g) || ensure_pinned(c, 16ull * ng))
         return;
     // (allocations on the context's stream; and no copy uses the pinned buffer)
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return;
     uint32_t *gidx = (uint32_t *)c->h_pin;
     for (uint32_t g = 0; g < ng; g++) gidx[g] = gidx[ng + g] = alone[gi[g]].slot;
+    memset(gidx + 2 * ng, 0, 8ull * ng);  // (the groups' release words)
     GroupArgs G{};
     G.slot = S->args.slot;
     G.prob = (const uint32_t *)c->g_idx.p;
     G.slot_of = (const uint32_t *)c->g_idx.p + ng;
+    G.release = (unsigned long long *)c->g_idx.p + ng;
     G.groups = ng;
     G.group_ctas = gctas;
     G.blk = (uint32_t *)c->g_blk.p;
@@ -2205,7 +2209,7 @@ void continue_in_slots(rei_server *S, std::vector<rei_server::Req> &alone) {
     G.bitmap = (uint32_t *)c->g_bitmap.p;
     G.chunk = chunk_g;
     G.tmp_words = tmp_g;
-    if (cudaMemcpyAsync(c->g_idx.p, gidx, 8ull * ng, cudaMemcpyHostToDevice, S->kstream) != cudaSuccess ||
+    if (cudaMemcpyAsync(c->g_idx.p, gidx, 16ull * ng, cudaMemcpyHostToDevice, S->kstream) != cudaSuccess ||
         cudaMemsetAsync(c->g_bitmap.p, 0, 4ull * ng * bmw_g, S->kstream) != cudaSuccess ||
         launch_solve_groups(S->args.parked, &G, ng * gctas, threads_g, smem_g, S->kstream) != cudaSuccess ||
         cudaStreamSynchronize(S->kstream) != cudaSuccess) {

@@ -292,6 +292,9 @@ struct GroupArgs {
     uint32_t *tmp, *pending, *slotpos, *bitmap;
     uint64_t chunk, tmp_words;
     uint64_t yield_ns;               // a search still running after this long parks again (0 = never)
+    // one word per group, zero before the launch: set once the group's first
+    // CTA has reset the slot's state, which the others read none of before
+    unsigned long long *release;
 };
 
 struct BatchArgs {

@@ -144,11 +144,16 @@ __global__ void __launch_bounds__(256, 2) k_solve_batch(const BatchJob *jobs, co
 // searches a batch left in their slots at their time allowance, continued side
 // by side: group g of G.group_ctas CTAs takes problem G.prob[g] in its slot and
 // runs the plain search there (its first CTA leads, the others take the team
-// chunks), with the slot's cache, uniqueness table and state as the batch CTA
-// left them.  The leader writes the problem's report like a batch CTA.
+// chunks), with the slot's cache, uniqueness table and state as the batch CTA,
+// or the group launch before, left them.  The leader writes the problem's report
+// like a batch CTA.  A slot that a group has parked holds that launch's last
+// command (to leave) and its barrier's arrivals: the leader resets them and then
+// releases the others, which wait for its word (the host zeroes it in the copy
+// that brings the groups, so it costs a batch nothing; the wait is bounded).
 __global__ void __launch_bounds__(256, 2) k_solve_groups(const BatchJob *jobs, const __grid_constant__ GroupArgs G) {
     __shared__ SolveJob J;
     __shared__ unsigned long long s_t0;
+    __shared__ uint32_t s_go;
     const uint32_t g = blockIdx.x / G.group_ctas;
     if (g >= G.groups) return;
     const uint32_t slot = G.slot_of[g];
@@ -174,10 +179,10 @@ __global__ void __launch_bounds__(256, 2) k_solve_groups(const BatchJob *jobs, c
         J.handover = 0;
         s_t0 = globaltimer_ns();
         J.t_start = s_t0;
-        // (the leader continues the parked search; the other CTAs read no
-        // state before its first command)
+        // the leader continues the parked search
+        SolveState *st = J.st;
+        uint32_t go = 1;
         if (team_rank_of(J) == 0) {
-            SolveState *st = J.st;
             st->status = ST_RUNNING;
             st->need_rows = 0;
             st->marked = 0;
@@ -185,9 +190,25 @@ __global__ void __launch_bounds__(256, 2) k_solve_groups(const BatchJob *jobs, c
             st->cmd = 0;
             st->cmd_seq = 0;
             st->err = 0;
+            __threadfence();
+            atomicExch(&G.release[g], 1ull);
+        } else {
+            uint32_t nap = 64;
+            while ((go = (uint32_t)ld_acquire_u64(&G.release[g])) == 0) {
+                if (globaltimer_ns() - s_t0 > kBarrierWaitNs) break;
+                __nanosleep(nap);
+                if (nap < REI_CMD_NAP) nap <<= 1;
+            }
+            if (!go) {
+                // (never released: the search ends with an error for the host)
+                atomicCAS(&st->err, 0u, 4u);
+                atomicExch(&st->status, (uint32_t)ST_TIMEOUT);
+            }
         }
+        s_go = go;
     }
     __syncthreads();
+    if (!s_go) return;
     uint32_t epoch = 0;
     solve_body<kAnyWidth, false>(J, epoch);
     if (team_rank_of(J) == 0 && threadIdx.x == 0)
