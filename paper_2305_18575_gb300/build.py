@@ -19,7 +19,9 @@ LIB = os.path.join(LIBDIR, "librei.so")
 PEAK_LIB = os.path.join(LIBDIR, "librei_peak.so")
 SOURCES = ["stage.cu", "solve.cu", "relaunch.cu", "slots.cu", "host.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
+# (device code stored as it is: with -lineinfo nvcc compresses it, and the first
+# relaunch of a process then waited 11 ms while 10.8 MB were unpacked; 1 ms so)
+FLAGS = ["-O3", "-lineinfo", "--compress-mode=none", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 
 
 def nvcc() -> str:
@@ -33,6 +35,7 @@ def _deps():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     files.append(os.path.join(os.path.dirname(HERE), "include", "rei.h"))
+    files.append(os.path.abspath(__file__))  # (the flags)
     return files
 
 
