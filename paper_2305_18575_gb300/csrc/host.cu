@@ -23,6 +23,7 @@
 #include "rei_dev.cuh"
 #include "stage_dev.cuh"
 #include "args.h"
+#include "sizes.h"
 
 namespace rei {
 cudaError_t launch_solve_batch(const BatchJob *jobs_dev, const BatchArgs *args, uint32_t grid, uint32_t threads,
@@ -207,12 +208,6 @@ rei_status ensure_pinned(rei_ctx *c, size_t bytes) {
 uint64_t budget_cap(uint64_t budget, uint32_t n) {
     const uint64_t per = 4ull * padded_words(n) + 28;
     return std::min<uint64_t>(budget / per, 0x7FFF0000ull);
-}
-
-uint64_t pow2_at_least(uint64_t x) {
-    uint64_t p = 1;
-    while (p < x) p <<= 1;
-    return p;
 }
 
 // ---------------------------------------------------------------------------
@@ -857,18 +852,10 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     const uint64_t cap_rows = n < 63 ? std::min<uint64_t>(cap, 1ull << n) : cap;
     cache_alloc = std::max<uint64_t>(1, std::min<uint64_t>(cache_alloc, cap_rows));
 
-    auto table_slots = [&](uint64_t alloc_rows) {
-        uint64_t need = alloc_rows + (alloc_rows >= cap ? chunk_max : 0);
-        // (the table holds distinct languages: at most 2^n of them; with
-        // 1-word exact keys up to 2^26 it has a slot for every language, the
-        // language itself, and is never probed twice)
-        if (n < 40) need = std::min<uint64_t>(need, 1ull << n);
-        return use_direct ? 1ull << n : pow2_at_least(std::max<uint64_t>(2 * need, 1024));
-    };
     // (exact keys: the language and its first candidate; else one word)
     const bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
     const uint64_t slot_bytes = exact_keys && !use_direct ? 16 : 8;
-    uint64_t tslots = table_slots(cache_alloc);
+    uint64_t tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
     // after a fused launch the cache holds its rows: grow keeping them
     auto ensure_rows = [&](DevBuf &b, size_t bytes) {
         return fused ? grow_keep(c, b, bytes, b.bytes) : ensure(c, b, bytes);
@@ -1037,7 +1024,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
         if ((s = grow_keep(c, c->bp_r, 4ull * want, 4ull * rows))) return s;
         if ((s = grow_keep(c, c->used, 4ull * want, 0))) return s;
         cache_alloc = want;
-        tslots = table_slots(cache_alloc);
+        tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
         {
             const void *before = c->table.p;
             if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;

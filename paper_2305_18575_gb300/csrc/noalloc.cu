@@ -29,6 +29,7 @@
 
 #include "rei_dev.cuh"
 #include "args.h"
+#include "sizes.h"
 
 namespace rei {
 cudaError_t launch_stage(const StageJob *jobs_dev, uint32_t n_jobs, cudaStream_t stream);
@@ -82,12 +83,6 @@ struct Carve {
         return base + at;
     }
 };
-
-uint64_t pow2_at_least(uint64_t x) {
-    uint64_t p = 1;
-    while (p < x) p <<= 1;
-    return p;
-}
 
 // postfix tokens -> pretty string, with fixed-size stack storage only
 size_t format_noalloc(const uint8_t *tok, uint32_t ntok, const uint8_t *alpha, char *out, size_t cap) {

@@ -1,0 +1,31 @@
+// sizes.h -- sizes of a search's buffers (host side).
+#pragma once
+#include <algorithm>
+#include <cstdint>
+
+namespace rei {
+
+inline uint64_t pow2_at_least(uint64_t x) {
+    uint64_t p = 1;
+    while (p < x) p <<= 1;
+    return p;
+}
+
+// A table slot's number is held in 32 bits: with a marked candidate, in the list
+// of slots a search empties, and in a candidate's registers.
+constexpr uint64_t kMaxTableSlots = 1ull << 32;
+
+// Slots of the uniqueness table of a search with room for `rows` languages of at
+// most `cap`: at most half full with them and, once the cache cannot grow, a
+// chunk of candidates that find no room.  It holds distinct languages, at most
+// 2^n of them; direct: a slot for every language (1-word exact keys up to 2^26,
+// never probed twice).  Bounded by the slots' numbers: 0x7FFF0000 languages and a
+// chunk of 2^26 fill 52 % of 2^32 slots.
+inline uint64_t table_slots(uint64_t rows, uint64_t cap, uint64_t chunk, uint32_t n, bool direct) {
+    if (direct) return 1ull << n;
+    uint64_t need = rows + (rows >= cap ? chunk : 0);
+    if (n < 40) need = std::min<uint64_t>(need, 1ull << n);
+    return std::min(kMaxTableSlots, pow2_at_least(std::max<uint64_t>(2 * need, 1024)));
+}
+
+}  // namespace rei

@@ -1,0 +1,58 @@
+"""Sizes of the uniqueness table (csrc/sizes.h), compiled for the host: at most
+2^32 slots, whose numbers the search holds in 32 bits, and room enough below that."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2305_18575_gb300", "csrc")
+CAP = 0x7FFF0000  # the most languages a cache holds
+MAIN = """
+#include <cstdio>
+#include <cstdlib>
+#include "sizes.h"
+int main(int argc, char **argv) {
+    for (int i = 1; i + 4 < argc; i += 5)
+        printf("%llu\\n", (unsigned long long)rei::table_slots(strtoull(argv[i], 0, 0), strtoull(argv[i + 1], 0, 0),
+               strtoull(argv[i + 2], 0, 0), (uint32_t)strtoull(argv[i + 3], 0, 0), atoi(argv[i + 4]) != 0));
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def table_slots(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("sizes")
+    (d / "main.cpp").write_text(MAIN)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(d / "main.cpp"), "-o", str(d / "main")], check=True)
+
+    def f(rows, cap, chunk, n, direct=0):
+        out = subprocess.run([str(d / "main"), *map(str, (rows, cap, chunk, n, direct))], check=True,
+                             capture_output=True, text=True)
+        return int(out.stdout)
+    return f
+
+
+@pytest.mark.parametrize("n", [27, 30, 31, 32, 33, 40, 62, 64, 129])
+@pytest.mark.parametrize("chunk", [1 << 16, 1 << 25, 1 << 26, 1 << 28])
+def test_the_largest_tables_slots_are_numbered_in_32_bits(table_slots, n, chunk):
+    for rows in (1 << 30, (1 << 30) + 1, CAP - 1, CAP):
+        rows = min(rows, 1 << n)
+        slots = table_slots(rows, CAP, chunk, n)
+        held = min(rows + (chunk if rows >= CAP else 0), 1 << min(n, 40))
+        assert slots & (slots - 1) == 0 and slots <= 1 << 32
+        # (half full, or the bound: some 1 - 6 % more)
+        assert held <= slots // 2 or (slots == 1 << 32 and held <= 0.57 * slots)
+
+
+def test_smaller_tables_are_at_most_half_full(table_slots):
+    assert table_slots(1, 10, 0, 62) == 1024
+    assert table_slots(65536, 1 << 20, 4096, 40) == 1 << 17
+    assert table_slots(1 << 20, 1 << 20, 4096, 40) == 1 << 22
+    assert table_slots(1 << 20, 1 << 20, 4096, 12) == 1 << 13
+    assert table_slots(5, 10, 4096, 26, direct=1) == 1 << 26
+    assert table_slots((1 << 30) + 1, CAP, 1 << 25, 40) == 1 << 32
