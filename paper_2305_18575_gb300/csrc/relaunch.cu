@@ -38,9 +38,9 @@ __global__ void k_rehash(const __grid_constant__ SolveJob J, uint32_t count) {
         } else {
             const uint64_t h = cs_hash(c, W, 1);
             const unsigned long long v = ((uint64_t)(uint32_t)(h >> 32) << 32) | (uint32_t)k;
-            uint64_t p = h & J.table_mask;
-            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = (p + 1) & J.table_mask;
-            J.used[k] = (uint32_t)p;
+            uint32_t p = probe_first(h, J.table_mask);
+            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = probe_next(p, (uint32_t)J.table_mask);
+            J.used[k] = p;
         }
         if (J.seen) atomicOr(J.seen + (c[0] >> 5), 1u << (c[0] & 31u));
     }

@@ -28,6 +28,7 @@
 #include <cstddef>
 
 #include "rei_dev.cuh"
+#include "sizes.h"
 #include "stage_dev.cuh"
 
 namespace rei {
@@ -472,9 +473,6 @@ struct TileCtx {
     bool reg;                   // binary tiles of 32 * reg_per candidates, built in registers
 };
 
-// no table slot: a candidate that is not marked
-constexpr uint32_t kNoMark = 0xFFFFFFFFu;
-
 // Language rows in global memory, compared with and written from a
 // candidate's words in shared memory.  Whole 16-byte loads, two of them in
 // flight before any is tested: the word-by-word compare with an early exit
@@ -611,7 +609,7 @@ __device__ void dedup_insert_solo(const TileCtx &T, const uint32_t *c, uint32_t 
     const uint64_t h = cs_hash(c, W, 1);
     const uint32_t fp = (uint32_t)(h >> 32);
     const unsigned long long mine = ((uint64_t)fp << 32) | kPending | xl;
-    uint64_t p = h & J.table_mask;
+    uint32_t p = probe_first(h, J.table_mask);
     row_write(J.tmp + (uint64_t)xl * W, c, W, T.vec);
     __threadfence_block();
     for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
@@ -634,7 +632,7 @@ __device__ void dedup_insert_solo(const TileCtx &T, const uint32_t *c, uint32_t 
                 return;
             }
         }
-        p = (p + 1) & J.table_mask;
+        p = probe_next(p, (uint32_t)J.table_mask);
     }
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
 }
@@ -667,7 +665,8 @@ __device__ __forceinline__ unsigned long long exact_key(const uint32_t *c, uint3
 
 // exact keys: the table slot a probe starts at.  The top bits of a
 // multiplicative hash (Knuth, "The Art of Computer Programming" 3, 6.4), an
-// even slot: the second probe then lies in the first one's 32-byte sector.
+// even slot: the second probe then lies in the first one's 32-byte sector (and
+// the last slot, kNoMark in the largest table, is never the first).
 __device__ __forceinline__ uint64_t exact_slot(const SolveJob &J, unsigned long long key) {
     if (J.direct) return key;
     const unsigned long long h = (key ^ (key >> 31)) * 0x9E3779B97F4A7C15ull;
@@ -677,9 +676,9 @@ __device__ __forceinline__ uint64_t exact_slot(const SolveJob &J, unsigned long 
 // a cached language into the table, with epoch 0 (languages that are all
 // distinct, while no other insertion runs); returns its slot
 __device__ __forceinline__ uint64_t exact_fill(const SolveJob &J, unsigned long long key, uint32_t row) {
-    uint64_t p = exact_slot(J, key);
+    uint32_t p = (uint32_t)exact_slot(J, key);
     if (!J.direct)
-        while (atomicCAS(&J.table[2 * p], kEmpty, key) != kEmpty) p = (p + 1) & J.table_mask;
+        while (atomicCAS(&J.table[2ull * p], kEmpty, key) != kEmpty) p = probe_next(p, (uint32_t)J.table_mask);
     *exact_meta(J, p) = row;
     return p;
 }
@@ -700,17 +699,17 @@ __device__ uint32_t dedup_insert_exact(const TileCtx &T, const uint32_t *c, uint
     // through L2).  Languages new in this chunk take the table protocol below.
     if (J.seen && ((ldcg(J.seen + (c[0] >> 5)) >> (c[0] & 31u)) & 1u)) return kNoMark;
     const unsigned long long key = exact_key(c, W), mine = exact_entry(T.epoch, xl);
-    uint64_t p = exact_slot(J, key);
+    uint32_t p = (uint32_t)exact_slot(J, key);
     for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
         unsigned long long v = key, m;
         if (J.direct) {
             m = ld_relaxed_u64(&J.table[p]);
         } else {
-            const ulonglong2 s = ld_relaxed_u64x2(&J.table[2 * p]);
+            const ulonglong2 s = ld_relaxed_u64x2(&J.table[2ull * p]);
             v = s.x;
             m = s.y;
             if (v == kEmpty) {
-                v = atomicCAS(&J.table[2 * p], kEmpty, key);
+                v = atomicCAS(&J.table[2ull * p], kEmpty, key);
                 if (v == kEmpty) v = key;
                 m = kEmpty;  // (whoever claimed it, its first candidate is of this chunk)
             }
@@ -723,9 +722,9 @@ __device__ uint32_t dedup_insert_exact(const TileCtx &T, const uint32_t *c, uint
                 T.ent[xl] = p;
                 atomicOr(&T.bits[xl >> 5], 1u << (xl & 31));
             }
-            return (uint32_t)p;
+            return p;
         }
-        p = (p + 1) & J.table_mask;
+        p = probe_next(p, (uint32_t)J.table_mask);
     }
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
     return kNoMark;
@@ -741,7 +740,7 @@ __device__ uint32_t dedup_insert(const TileCtx &T, const uint32_t *c, uint32_t x
     const uint64_t h = cs_hash(c, W, 1);
     const uint32_t fp = (uint32_t)(h >> 32);
     const uint64_t mine = ((uint64_t)fp << 32) | kPending | xl;
-    uint64_t p = h & J.table_mask;
+    uint32_t p = probe_first(h, J.table_mask);
     bool wrote = false;
     auto write_tmp = [&]() {
         if (wrote) return;
@@ -772,7 +771,7 @@ __device__ uint32_t dedup_insert(const TileCtx &T, const uint32_t *c, uint32_t x
                 return (uint32_t)p;
             }
         }
-        p = (p + 1) & J.table_mask;
+        p = probe_next(p, (uint32_t)J.table_mask);
     }
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
     return kNoMark;
@@ -1314,7 +1313,7 @@ __device__ __forceinline__ void w2_finish(const TileCtx &T, const Seg &sg, const
                     }
                     act &= ~(1u << k);
                 } else {
-                    p[k] = (p[k] + 1) & (uint32_t)J.table_mask;
+                    p[k] = probe_next(p[k], (uint32_t)J.table_mask);
                 }
             }
             if (++rounds > J.table_mask) {
@@ -1835,8 +1834,8 @@ __device__ inline void switch_to_global(const SolveJob &J, Shared &S, Lead *L) {
         } else {
             const uint64_t h = cs_hash(row, W, 1);
             const unsigned long long v = ((uint64_t)(uint32_t)(h >> 32) << 32) | k;
-            uint64_t p = h & J.table_mask;
-            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = (p + 1) & J.table_mask;
+            uint32_t p = probe_first(h, J.table_mask);
+            while (atomicCAS(&J.table[p], kEmpty, v) != kEmpty) p = probe_next(p, (uint32_t)J.table_mask);
             J.used[k] = (uint32_t)p;
         }
         if (J.seen) atomicOr(J.seen + (row[0] >> 5), 1u << (row[0] & 31u));

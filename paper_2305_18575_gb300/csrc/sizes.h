@@ -1,7 +1,14 @@
-// sizes.h -- sizes of a search's buffers (host side).
+// sizes.h -- sizes of a search's buffers, and the slots of its uniqueness table in
+// the order they are probed (host and device).
 #pragma once
 #include <algorithm>
 #include <cstdint>
+
+#ifdef __CUDACC__
+#define REI_HD __host__ __device__ __forceinline__
+#else
+#define REI_HD inline
+#endif
 
 namespace rei {
 
@@ -14,6 +21,20 @@ inline uint64_t pow2_at_least(uint64_t x) {
 // A table slot's number is held in 32 bits: with a marked candidate, in the list
 // of slots a search empties, and in a candidate's registers.
 constexpr uint64_t kMaxTableSlots = 1ull << 32;
+
+// Linear probing of a table of mask + 1 slots from hash h.  No candidate is marked
+// with slot kNoMark, the last of the largest table: the number says that a candidate
+// is not marked, and probing passes the slot over.  (A flag beside the slot instead
+// cost 12-word searches 2 %, medium ones 0.5 %.)
+constexpr uint32_t kNoMark = 0xFFFFFFFFu;
+REI_HD uint32_t probe_first(uint64_t h, uint64_t mask) {
+    const uint32_t p = (uint32_t)(h & mask);
+    return p < kNoMark - 1 ? p : kNoMark - 1;
+}
+REI_HD uint32_t probe_next(uint32_t p, uint32_t mask) {
+    const uint32_t q = (p + 1) & mask;
+    return q == kNoMark ? 0u : q;
+}
 
 // Slots of the uniqueness table of a search with room for `rows` languages of at
 // most `cap`: at most half full with them and, once the cache cannot grow, a

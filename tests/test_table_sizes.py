@@ -56,3 +56,40 @@ def test_smaller_tables_are_at_most_half_full(table_slots):
     assert table_slots(1 << 20, 1 << 20, 4096, 12) == 1 << 13
     assert table_slots(5, 10, 4096, 26, direct=1) == 1 << 26
     assert table_slots((1 << 30) + 1, CAP, 1 << 25, 40) == 1 << 32
+
+
+PROBE = """
+#include <cstdio>
+#include "sizes.h"
+int main() {
+    using rei::probe_first;
+    using rei::probe_next;
+    const uint64_t top = 0xFFFFFFFFull;
+    // the largest table: its last slot is passed over, from either side
+    if (probe_first(0x12345678FFFFFFFFull, top) != top - 1 || probe_first(0x12345678FFFFFFFEull, top) != top - 1) return 1;
+    if (probe_next(0xFFFFFFFEu, 0xFFFFFFFFu) != 0 || probe_next(0xFFFFFFFDu, 0xFFFFFFFFu) != 0xFFFFFFFEu) return 2;
+    if (probe_next(7u, 0xFFFFFFFFu) != 8) return 3;
+    // any other: every slot in turn
+    for (uint64_t bits = 10; bits < 32; bits++) {
+        const uint64_t mask = (1ull << bits) - 1;
+        const uint32_t m = (uint32_t)mask;
+        if (probe_first(~0ull, mask) != mask || probe_first(~0ull - 1, mask) != mask - 1) return 4;
+        if (probe_next(m - 1, m) != m || probe_next(m, m) != 0) return 5;
+    }
+    return 0;
+}
+"""
+
+
+def test_probing_passes_over_the_number_that_means_not_marked(tmp_path):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no g++")
+    (tmp_path / "probe.cpp").write_text(PROBE)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(tmp_path / "probe.cpp"), "-o", str(tmp_path / "probe")], check=True)
+    assert subprocess.run([str(tmp_path / "probe")]).returncode == 0
+    # and nothing in the searches probes by itself
+    for name in ("search.cuh", "relaunch.cu", "slots.cu", "solve.cu"):
+        with open(os.path.join(CSRC, name)) as fh:
+            text = fh.read()
+        assert "+ 1) & J.table_mask" not in text and "h & J.table_mask" not in text, name
