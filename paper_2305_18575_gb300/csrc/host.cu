@@ -40,6 +40,7 @@ cudaError_t launch_solve(const SolveJob *job, uint32_t grid, uint32_t threads, s
                          cudaStream_t stream);
 cudaError_t solve_occupancy(uint32_t W, uint32_t threads, size_t smem, int *blocks_per_sm);
 cudaError_t solve_smem_max(uint32_t W, size_t *bytes);
+uint32_t solve_warps_max(uint32_t W);  // warps a CTA of this width's relaunch can have
 cudaError_t solve_batch_smem_max(size_t *bytes);
 cudaError_t launch_solve_groups(const BatchJob *jobs_dev, const GroupArgs *args, uint32_t grid, uint32_t threads,
                                 size_t smem, cudaStream_t stream);
@@ -79,7 +80,7 @@ struct rei_ctx {
     int64_t opt_chunk = 0, opt_grid = 0, opt_keep = 0, opt_cache_init = 0, opt_solo_tiles = -1, opt_small_rows = -1;
     int64_t opt_fused = 1, opt_exact = 1;
     uint64_t opt_handover = 1ull << 22;  // levels of more candidates leave the fused launch
-    uint32_t share = 1;                  // this context's relaunches take one in `share` of the GPU's SMs
+    uint32_t share = 1;                  // launches side by side: each has CTAs for one in `share` of the GPU's SMs
     uint64_t opt_yield_us = 500;         // batched / served problems longer than this continue on the whole GPU
     bool phases = getenv("REI_PHASES") != nullptr;  // per-solve timing report on stderr (diagnostics)
     unsigned long long fused_launch_id = 0;         // ids of this context's fused launches (only grow)
@@ -786,7 +787,9 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     size_t smem_max = 0;  // dynamic shared memory a k_solve launch can take
     CK(solve_smem_max(W, &smem_max));
     bool gt_smem = 4ull * (n + 1 + G + max_len + 2) <= 96 * 1024;
-    uint32_t warps = 16;  // (the launch bounds of k_solve)
+    // 16 warps a CTA, or beside other launches as many as fill an SM alone (below)
+    const uint32_t warps_top = c->share > 1 ? solve_warps_max(W) : 16;
+    uint32_t warps = warps_top;
     size_t smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps);
     while (smem > smem_max && warps > 1) {
         warps /= 2;
@@ -794,7 +797,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     }
     if (smem > smem_max && gt_smem) {
         gt_smem = false;
-        warps = 16;
+        warps = warps_top;
         smem = solve_smem_bytes(W, n, G, max_len, seg_cap, gt_smem, warps);
         while (smem > smem_max && warps > 1) {
             warps /= 2;
@@ -823,9 +826,13 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     int bps = 0;
     CK(solve_occupancy(W, threads, smem, &bps));
     if (bps < 1) return REI_ECUDA;
-    // (a helper's launch takes its share of the SMs, whatever CTAs of this
-    // width fit one: launches side by side whose CTAs wait for each other must
-    // fit the GPU together)
+    // Launches side by side, whose CTAs wait for each other, must fit the GPU
+    // together wherever the CTAs of the others lie (one that takes half an SM
+    // keeps a launch that needs whole ones off it): together they have at most one
+    // CTA an SM, so that one not yet placed always finds an SM of its own.  CTAs
+    // of 32 warps where two of 16 would fit (eight searches of 1-word languages
+    // that outgrew their slots: 5.6 ms a batch; with 16 warps 6.6 ms)
+    if (c->share > 1) bps = 1;
     grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
     if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
 

@@ -12,8 +12,11 @@ namespace rei {
 // L1, 9.4 ms; 1-word languages, bound by the L2, lost a tenth with one, 4-word
 // ones a sixth), and from 20 words on, where the warps' tiles leave room for one
 // CTA an SM anyway (32 words to cost 12: 9.1 -> 8.0 ms; 12 words lost a fifth).
+// The two CTAs may also be one of 32 warps: searches side by side take one an SM
+// (solve_warps_max).
 template <uint32_t WC>
-__global__ void __launch_bounds__(kSolveThreads, WC == kWidest || WC == 2 ? 1 : 2) k_solve(const __grid_constant__ SolveJob J) {
+__global__ void __launch_bounds__(WC == kWidest || WC == 2 ? kSolveThreads : 2 * kSolveThreads, 1)
+    k_solve(const __grid_constant__ SolveJob J) {
     uint32_t bar_epoch = 0;
     solve_body<WC>(J, bar_epoch);
 }
@@ -60,6 +63,8 @@ cudaError_t solve_occupancy(uint32_t W, uint32_t threads, size_t smem, int *bloc
 }
 
 cudaError_t solve_smem_max(uint32_t W, size_t *bytes) { return smem_max_of(solve_kernel(W), bytes); }
+
+uint32_t solve_warps_max(uint32_t W) { return (W == 2 || W >= kWidest ? 1 : 2) * kSolveThreads / 32; }
 
 cudaError_t launch_rehash(const SolveJob *job, uint32_t count, uint32_t grid, cudaStream_t stream) {
     k_rehash<<<grid, 256, 0, stream>>>(*job, count);
