@@ -46,6 +46,12 @@
  *     without yielding an answer ends the search with REI_OOM, or, with
  *     REI_F_ONTHEFLY, continues uncached while every operand level it needs
  *     is complete ("OnTheFly mode", Sec. 3).
+ *     The budget counts the languages.  The uniqueness table comes on top of
+ *     it: two to four slots for each language the cache has room for (at most
+ *     2^32), of 16 bytes for |ic| 27 to 62 (the language and its first
+ *     candidate) and of 8 bytes otherwise or where 16 do not fit the device
+ *     (fingerprints); 2^|ic| slots of 8 bytes for |ic| <= 26.  So do a chunk's
+ *     lists (8 bytes and a bit a candidate) and, with fingerprints, its rows.
  */
 #ifndef REI_H
 #define REI_H

@@ -139,7 +139,10 @@ void *dev_alloc(rei_ctx *c, size_t bytes) {
     if (bytes == 0) bytes = 16;
     void *p = nullptr;
     if (c->has_alloc) return c->alloc.alloc(c->alloc.user, bytes, (void *)c->stream);
-    if (cudaMallocAsync(&p, bytes, c->stream) != cudaSuccess) return nullptr;
+    if (cudaMallocAsync(&p, bytes, c->stream) != cudaSuccess) {
+        cudaGetLastError();  // (reported to the caller, not by a later launch)
+        return nullptr;
+    }
     return p;
 }
 
@@ -186,6 +189,13 @@ rei_status clear_table(rei_ctx *c, uint64_t at_least) {
     if (t) CK(cudaMemsetAsync(c->table.p, 0xFF, t, c->stream));
     c->table_extent = 0;
     return REI_OK;
+}
+
+// The table given back: the next one allocated holds garbage.
+void drop_table(rei_ctx *c) {
+    dev_free(c, c->table);
+    c->table_clean = false;
+    c->table_extent = 0;
 }
 
 rei_status ensure_pinned(rei_ctx *c, size_t bytes) {
@@ -490,32 +500,8 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
         rows = std::max<uint64_t>(rows, std::min<uint64_t>(have, 1ull << 20));
     }
     const uint64_t wguess = std::max<uint32_t>(2u, c->last_W);
-    if ((s = ensure(c, c->cs, 4ull * wguess * rows))) return s;
-    if ((s = ensure(c, c->bp_op, rows))) return s;
-    if ((s = ensure(c, c->bp_l, 4ull * rows))) return s;
-    if ((s = ensure(c, c->bp_r, 4ull * rows))) return s;
-    if ((s = ensure(c, c->used, 4ull * rows))) return s;
     const uint64_t tslots = pow2_at_least(std::max<uint64_t>(4 * rows, 1024));
-    {
-        // a reallocated table (even at the same address) holds garbage
-        const void *before = c->table.p;
-        const size_t before_bytes = c->table.bytes;
-        if ((s = ensure(c, c->table, 16ull * tslots))) return s;
-        if (c->table.p != before || c->table.bytes != before_bytes) {
-            c->table_clean = false;
-            c->table_extent = c->table.bytes;
-        }
-    }
     const uint64_t chunk_words = c->opt_chunk > 0 ? (uint64_t)c->opt_chunk : (1ull << 22);
-    if ((s = ensure(c, c->tmp, std::max<uint64_t>(4ull * 2 * chunk_words, 4ull * 64 * 4096)))) return s;
-    if ((s = ensure(c, c->pending, 4ull * chunk_words))) return s;
-    if ((s = ensure(c, c->slotpos, 4ull * chunk_words))) return s;
-    {
-        const void *before = c->bitmap.p;
-        const size_t before_bytes = c->bitmap.bytes;
-        if ((s = ensure(c, c->bitmap, 4ull * ((chunk_words + 31) / 32)))) return s;
-        if (c->bitmap.p != before || c->bitmap.bytes != before_bytes) c->table_clean = false;
-    }
     const uint32_t threads = 512;  // (the launch bounds of k_solve_fused: one 16-warp CTA per SM)
     const size_t smem = c->smem_optin > 8192 ? c->smem_optin - 8192 : 0;  // (its static shared memory and a reserve)
     int bps = 0;
@@ -523,31 +509,70 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     if (bps < 1) return REI_EBUSY;
     uint32_t grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
     if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
-    if ((s = ensure(c, c->blk, 4ull * grid))) return s;
-    if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
-    if ((s = ensure(c, c->lvl_count, 8ull * (max_cost + 2)))) return s;
-    {
-        // a new state buffer starts zeroed: the launch id it holds is then
-        // always below the next launch's (the launch resets the rest itself)
-        const void *before = c->state.p;
-        if ((s = ensure(c, c->state, sb + sizeof(StageInfo)))) return s;
-        if (c->state.p != before) CK(cudaMemsetAsync(c->state.p, 0, c->state.bytes, c->stream));
+    bool exact = c->opt_exact != 0;  // allowed; the launch decides from the staged size
+    uint64_t slot_bytes = 16;
+    auto buffers = [&]() -> rei_status {
+        rei_status s;
+        if ((s = ensure(c, c->cs, 4ull * wguess * rows))) return s;
+        if ((s = ensure(c, c->bp_op, rows))) return s;
+        if ((s = ensure(c, c->bp_l, 4ull * rows))) return s;
+        if ((s = ensure(c, c->bp_r, 4ull * rows))) return s;
+        if ((s = ensure(c, c->used, 4ull * rows))) return s;
+        {
+            // a reallocated table (even at the same address) holds garbage
+            const void *before = c->table.p;
+            const size_t before_bytes = c->table.bytes;
+            if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
+            if (c->table.p != before || c->table.bytes != before_bytes) {
+                c->table_clean = false;
+                c->table_extent = c->table.bytes;
+            }
+        }
+        if ((s = ensure(c, c->tmp, std::max<uint64_t>(4ull * 2 * chunk_words, 4ull * 64 * 4096)))) return s;
+        if ((s = ensure(c, c->pending, 4ull * chunk_words))) return s;
+        if ((s = ensure(c, c->slotpos, 4ull * chunk_words))) return s;
+        {
+            const void *before = c->bitmap.p;
+            const size_t before_bytes = c->bitmap.bytes;
+            if ((s = ensure(c, c->bitmap, 4ull * ((chunk_words + 31) / 32)))) return s;
+            if (c->bitmap.p != before || c->bitmap.bytes != before_bytes) c->table_clean = false;
+        }
+        if ((s = ensure(c, c->blk, 4ull * grid))) return s;
+        if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
+        if ((s = ensure(c, c->lvl_count, 8ull * (max_cost + 2)))) return s;
+        {
+            // a new state buffer starts zeroed: the launch id it holds is then
+            // always below the next launch's (the launch resets the rest itself)
+            const void *before = c->state.p;
+            if ((s = ensure(c, c->state, sb + sizeof(StageInfo)))) return s;
+            if (c->state.p != before) CK(cudaMemsetAsync(c->state.p, 0, c->state.bytes, c->stream));
+        }
+        if ((s = ensure(c, c->solve_job, sizeof(SolveJob)))) return s;
+        if ((s = ensure(c, c->tstack, 16ull * (max_cost + 2)))) return s;
+        if ((s = ensure(c, c->trace, 4ull * grid))) return s;
+        if ((s = ensure(c, c->plan, 8 * plan_words(2 * max_cost + 4)))) return s;
+        if (exact && !c->seen.p) {
+            if ((s = ensure(c, c->seen, (1ull << kSeenBits) / 8))) return s;
+            c->table_clean = false;
+        }
+        return REI_OK;
+    };
+    s = buffers();
+    if (s == REI_OOM) {
+        // (the relaunch's rule, see solve_one: fingerprints in half the table)
+        drop_table(c);
+        exact = false;
+        slot_bytes = 8;
+        s = buffers();
     }
-    if ((s = ensure(c, c->solve_job, sizeof(SolveJob)))) return s;
-    if ((s = ensure(c, c->tstack, 16ull * (max_cost + 2)))) return s;
-    if ((s = ensure(c, c->trace, 4ull * grid))) return s;
-    if ((s = ensure(c, c->plan, 8 * plan_words(2 * max_cost + 4)))) return s;
-    if (c->opt_exact && !c->seen.p) {
-        if ((s = ensure(c, c->seen, (1ull << kSeenBits) / 8))) return s;
-        c->table_clean = false;
-    }
+    if (s) return s;
     if (!c->table_clean) {
         if ((s = clear_table(c, 0))) return s;
         CK(cudaMemsetAsync(c->bitmap.p, 0, c->bitmap.bytes, c->stream));
         if (c->seen.p) CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
     }
     c->table_clean = false;
-    c->table_extent = std::max(c->table_extent, 16 * tslots);
+    c->table_extent = std::max(c->table_extent, slot_bytes * tslots);
 
     FuseArgs F;
     memset(&F, 0, sizeof F);
@@ -594,7 +619,7 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     j.used = (uint32_t *)c->used.p;
     j.table = (unsigned long long *)c->table.p;
     j.table_mask = tslots - 1;
-    j.exact = c->opt_exact ? 1u : 0u;  // allowed; the launch decides from the staged size
+    j.exact = exact ? 1u : 0u;
     j.tmp = (uint32_t *)c->tmp.p;
     j.pending = (uint32_t *)c->pending.p;
     j.slotpos = (uint32_t *)c->slotpos.p;
@@ -779,7 +804,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
 
     // 1-word languages with exact keys: a bitmap of the cached languages in
     // front of the uniqueness table
-    const bool use_seen = c->opt_exact && W == 1 && n <= kSeenBits;
+    bool use_seen = c->opt_exact && W == 1 && n <= kSeenBits;
     const bool use_direct = c->opt_exact && W == 1 && n <= kDirectBits;
 
     // launch shape
@@ -859,20 +884,15 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     const uint64_t cap_rows = n < 63 ? std::min<uint64_t>(cap, 1ull << n) : cap;
     cache_alloc = std::max<uint64_t>(1, std::min<uint64_t>(cache_alloc, cap_rows));
 
-    // (exact keys: the language and its first candidate; else one word)
-    const bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
-    const uint64_t slot_bytes = exact_keys && !use_direct ? 16 : 8;
-    uint64_t tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
-    // after a fused launch the cache holds its rows: grow keeping them
-    auto ensure_rows = [&](DevBuf &b, size_t bytes) {
-        return fused ? grow_keep(c, b, bytes, b.bytes) : ensure(c, b, bytes);
-    };
-    if ((s = ensure_rows(c->cs, 4ull * W * cache_alloc))) return s;
-    if ((s = ensure_rows(c->bp_op, cache_alloc))) return s;
-    if ((s = ensure_rows(c->bp_l, 4ull * cache_alloc))) return s;
-    if ((s = ensure_rows(c->bp_r, 4ull * cache_alloc))) return s;
-    if ((s = ensure(c, c->used, 4ull * cache_alloc))) return s;  // (rebuilt with the table)
-    {
+    bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
+    uint64_t tslots = 0, slot_bytes = 0;
+    // the table of cache_alloc rows, and the candidate rows, which wait in tmp only
+    // when the keys are fingerprints
+    auto ensure_table = [&]() -> rei_status {
+        rei_status s;
+        // (exact keys: the language and its first candidate; else one word)
+        slot_bytes = exact_keys && !use_direct ? 16 : 8;
+        tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
         const void *before = c->table.p;
         const size_t before_bytes = c->table.bytes;
         if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
@@ -880,40 +900,71 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
             c->table_clean = false;
             c->table_extent = c->table.bytes;
         }
-    }
-    // (candidate rows wait in tmp only when the keys are fingerprints)
-    if ((s = ensure(c, c->tmp, exact_keys ? 4096 : 4ull * W * chunk_max))) return s;
-    if ((s = ensure(c, c->pending, 4ull * chunk_max))) return s;
-    if ((s = ensure(c, c->slotpos, 4ull * chunk_max))) return s;
-    {
-        // a reallocated bitmap holds garbage: the search needs it zero
-        const void *before = c->bitmap.p;
-        const size_t before_bytes = c->bitmap.bytes;
-        if ((s = ensure(c, c->bitmap, 4ull * ((chunk_max + 31) / 32)))) return s;
-        if (c->bitmap.p != before || c->bitmap.bytes != before_bytes) {
-            if (fused) CK(cudaMemsetAsync(c->bitmap.p, 0, c->bitmap.bytes, c->stream));
-            else c->table_clean = false;
+        return ensure(c, c->tmp, exact_keys ? 4096 : 4ull * W * chunk_max);
+    };
+    // What to do when memory runs out: give back the table (it may be larger than
+    // this search's), and where a slot would be two words go on with one, that is
+    // with fingerprints, in chunks whose rows take half a word a slot at most.  So no
+    // search takes more memory than exact keys would in slots of 12 bytes.
+    auto smaller_table = [&]() -> rei_status {
+        drop_table(c);
+        if (!exact_keys || use_direct) return REI_OK;
+        if (use_seen && c->seen.p) CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
+        exact_keys = use_seen = false;
+        chunk_max = std::min(chunk_max, std::max<uint64_t>(1, table_slots(cache_alloc, cap, chunk_max, n, false) / W));
+        return REI_OK;
+    };
+    // after a fused launch the cache holds its rows: grow keeping them
+    auto ensure_rows = [&](DevBuf &b, size_t bytes) {
+        return fused ? grow_keep(c, b, bytes, b.bytes) : ensure(c, b, bytes);
+    };
+    auto buffers = [&]() -> rei_status {
+        rei_status s;
+        if ((s = ensure_rows(c->cs, 4ull * W * cache_alloc))) return s;
+        if ((s = ensure_rows(c->bp_op, cache_alloc))) return s;
+        if ((s = ensure_rows(c->bp_l, 4ull * cache_alloc))) return s;
+        if ((s = ensure_rows(c->bp_r, 4ull * cache_alloc))) return s;
+        if ((s = ensure(c, c->used, 4ull * cache_alloc))) return s;  // (rebuilt with the table)
+        if ((s = ensure_table())) return s;
+        if ((s = ensure(c, c->pending, 4ull * chunk_max))) return s;
+        if ((s = ensure(c, c->slotpos, 4ull * chunk_max))) return s;
+        {
+            // a reallocated bitmap holds garbage: the search needs it zero
+            const void *before = c->bitmap.p;
+            const size_t before_bytes = c->bitmap.bytes;
+            if ((s = ensure(c, c->bitmap, 4ull * ((chunk_max + 31) / 32)))) return s;
+            if (c->bitmap.p != before || c->bitmap.bytes != before_bytes) {
+                if (fused) CK(cudaMemsetAsync(c->bitmap.p, 0, c->bitmap.bytes, c->stream));
+                else c->table_clean = false;
+            }
         }
+        if ((s = ensure(c, c->blk, 4ull * grid))) return s;
+        if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
+        if ((s = ensure(c, c->lvl_count, 8ull * (max_cost + 2)))) return s;
+        {
+            const void *before = c->state.p;  // (a new state buffer starts zeroed, as in run_fused)
+            if ((s = ensure(c, c->state, sizeof(SolveState) + tree_bytes))) return s;
+            if (c->state.p != before) CK(cudaMemsetAsync(c->state.p, 0, c->state.bytes, c->stream));
+        }
+        if ((s = ensure(c, c->solve_job, sizeof(SolveJob)))) return s;
+        if ((s = ensure(c, c->tstack, 16ull * (max_cost + 2)))) return s;
+        if ((s = ensure(c, c->trace, 4ull * grid))) return s;
+        if ((s = ensure(c, c->plan, 8 * plan_words(seg_cap)))) return s;
+        if (use_seen && !c->seen.p) {
+            if ((s = ensure(c, c->seen, (1ull << kSeenBits) / 8))) return s;
+            CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
+        }
+        return REI_OK;
+    };
+    s = buffers();
+    if (s == REI_OOM) {
+        if ((s = smaller_table())) return s;
+        s = buffers();
     }
-    if ((s = ensure(c, c->blk, 4ull * grid))) return s;
-    if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
-    if ((s = ensure(c, c->lvl_count, 8ull * (max_cost + 2)))) return s;
-    {
-        const void *before = c->state.p;  // (a new state buffer starts zeroed, as in run_fused)
-        if ((s = ensure(c, c->state, sizeof(SolveState) + tree_bytes))) return s;
-        if (c->state.p != before) CK(cudaMemsetAsync(c->state.p, 0, c->state.bytes, c->stream));
-    }
-    if ((s = ensure(c, c->solve_job, sizeof(SolveJob)))) return s;
-    if ((s = ensure(c, c->tstack, 16ull * (max_cost + 2)))) return s;
-    if ((s = ensure(c, c->trace, 4ull * grid))) return s;
-    if ((s = ensure(c, c->plan, 8 * plan_words(seg_cap)))) return s;
+    if (s) return s;
     if ((s = ensure_pinned(c, sizeof(SolveJob) + sizeof(SolveState) + tree_bytes))) return s;
     hst = (SolveState *)(c->h_pin + sizeof(SolveJob));  // (the pinned buffer may have moved)
 
-    if (use_seen && !c->seen.p) {
-        if ((s = ensure(c, c->seen, (1ull << kSeenBits) / 8))) return s;
-        CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
-    }
     if (!fused) {
         if (!c->table_clean) {
             // a new table, or the last search ended abnormally: clear it once
@@ -975,7 +1026,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
         hj->used = (uint32_t *)c->used.p;
         hj->cache_alloc = cache_alloc;
         hj->table = (unsigned long long *)c->table.p;
-        hj->exact = (W <= 2 && n <= 62 && c->opt_exact) ? 1u : 0u;
+        hj->exact = exact_keys ? 1u : 0u;
         hj->seen = use_seen ? (uint32_t *)c->seen.p : nullptr;
         hj->direct = use_direct && tslots >= (1ull << n) ? 1u : 0u;
         hj->table_mask = tslots - 1;
@@ -1025,18 +1076,22 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
                                   ? std::min<uint64_t>(cap_rows, std::max<uint64_t>(cache_alloc * 4, hst->need_rows))
                                   : cache_alloc;
         const uint64_t rows = hst->size;
-        if ((s = grow_keep(c, c->cs, 4ull * W * want, 4ull * W * rows))) return s;
-        if ((s = grow_keep(c, c->bp_op, want, rows))) return s;
-        if ((s = grow_keep(c, c->bp_l, 4ull * want, 4ull * rows))) return s;
-        if ((s = grow_keep(c, c->bp_r, 4ull * want, 4ull * rows))) return s;
-        if ((s = grow_keep(c, c->used, 4ull * want, 0))) return s;
         cache_alloc = want;
-        tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
-        {
-            const void *before = c->table.p;
-            if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
-            if (c->table.p != before) c->table_extent = c->table.bytes;
+        auto grow = [&]() -> rei_status {
+            rei_status s;
+            if ((s = grow_keep(c, c->cs, 4ull * W * want, 4ull * W * rows))) return s;
+            if ((s = grow_keep(c, c->bp_op, want, rows))) return s;
+            if ((s = grow_keep(c, c->bp_l, 4ull * want, 4ull * rows))) return s;
+            if ((s = grow_keep(c, c->bp_r, 4ull * want, 4ull * rows))) return s;
+            if ((s = grow_keep(c, c->used, 4ull * want, 0))) return s;
+            return ensure_table();
+        };
+        s = grow();
+        if (s == REI_OOM) {
+            if ((s = smaller_table())) return s;
+            s = grow();
         }
+        if (s) return s;
         if ((s = clear_table(c, slot_bytes * tslots))) return s;  // (the rehash refills it)
         c->table_extent = slot_bytes * tslots;
         fill_job();
