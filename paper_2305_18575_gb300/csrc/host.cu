@@ -1915,10 +1915,13 @@ rei_status rei_solve_batch(rei_ctx *c, const rei_problem *probs, uint32_t n, rei
         struct Trial {
             uint32_t warps, chunk;
         };
+        // (a field that is given is tried as it is given)
+        const std::vector<uint32_t> try_warps = warps ? std::vector<uint32_t>{warps} : std::vector<uint32_t>{8, 4};
+        const std::vector<uint32_t> try_chunks =
+            chunk ? std::vector<uint32_t>{chunk} : std::vector<uint32_t>{1u << 11, 1u << 12, 1u << 14};
         std::vector<Trial> trials;
-        for (uint32_t w : {8u, 4u})
-            for (uint32_t ch : {1u << 11, 1u << 12, 1u << 14})
-                if ((!warps || w == warps) && (!chunk || ch == chunk)) trials.push_back({w, ch});
+        for (uint32_t w : try_warps)
+            for (uint32_t ch : try_chunks) trials.push_back({w, ch});
         Trial best{warps ? warps : 8u, chunk ? chunk : (1u << 11)};
         const size_t sample = (size_t)std::max(1, c->sm_count);
         double best_rate = -1;
