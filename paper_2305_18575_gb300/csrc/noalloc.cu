@@ -45,7 +45,6 @@ using namespace rei;
 
 namespace {
 
-constexpr size_t kAlign = 256;
 constexpr size_t kInputBytes = 1u << 20;      // example bytes
 constexpr uint32_t kMaxStrings = 1u << 16;    // examples (offsets table)
 constexpr uint32_t kPairCap = 1u << 18;       // guide-table pairs
@@ -71,18 +70,6 @@ cudaError_t scratch_address(int device, unsigned char **out) {
     *out = g_scratch_dev[device];
     return cudaSuccess;
 }
-
-// bump carving of the scratch array
-struct Carve {
-    unsigned char *base;
-    size_t used, cap;
-    void *take(size_t bytes) {
-        const size_t at = (used + kAlign - 1) & ~(kAlign - 1);
-        if (at + bytes > cap) return nullptr;
-        used = at + bytes;
-        return base + at;
-    }
-};
 
 // postfix tokens -> pretty string, with fixed-size stack storage only
 size_t format_noalloc(const uint8_t *tok, uint32_t ntok, const uint8_t *alpha, char *out, size_t cap) {

@@ -2,6 +2,7 @@
 // the order they are probed (host and device).
 #pragma once
 #include <algorithm>
+#include <cstddef>
 #include <cstdint>
 
 #ifdef __CUDACC__
@@ -21,6 +22,22 @@ inline uint64_t pow2_at_least(uint64_t x) {
 // A table slot's number is held in 32 bits: with a marked candidate, in the list
 // of slots a search empties, and in a candidate's registers.
 constexpr uint64_t kMaxTableSlots = 1ull << 32;
+
+// Bump carving of a fixed array.  A piece that does not fit ends it: the pieces after
+// it are refused too, whatever their size, so that the last of several tells of all.
+struct Carve {
+    static constexpr size_t kAlign = 256;
+    unsigned char *base;
+    size_t used, cap;
+    bool full = false;
+    void *take(size_t bytes) {
+        const size_t at = (used + kAlign - 1) & ~(kAlign - 1);
+        full = full || at > cap || bytes > cap - at;
+        if (full) return nullptr;
+        used = at + bytes;
+        return base + at;
+    }
+};
 
 // Linear probing of a table of mask + 1 slots from hash h.  No candidate is marked
 // with slot kNoMark, the last of the largest table: the number says that a candidate
