@@ -139,8 +139,9 @@ typedef struct rei_result {
     rei_stats stats;
 } rei_result;
 
-/* Optional device allocator.  alloc returns NULL on failure.  Both get the
- * context stream; the library frees everything it allocated before
+/* Optional device allocator.  alloc returns memory at an 8-byte boundary (at a
+ * 16-byte one the uniqueness table can hold exact keys, see above), or NULL on
+ * failure.  Both get the context stream; the library frees everything it allocated before
  * rei_ctx_destroy returns. */
 typedef struct rei_alloc {
     void *(*alloc)(void *user, size_t bytes, void *stream);

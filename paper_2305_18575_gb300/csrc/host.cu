@@ -191,6 +191,10 @@ rei_status clear_table(rei_ctx *c, uint64_t at_least) {
     return REI_OK;
 }
 
+// Slots of two words are read whole, so the table must lie at a 16-byte boundary;
+// an allocator of the caller's may give less.
+bool two_word_slots_fit(const rei_ctx *c) { return ((uintptr_t)c->table.p & 15) == 0; }
+
 // The table given back: the next one allocated holds garbage.
 void drop_table(rei_ctx *c) {
     dev_free(c, c->table);
@@ -566,6 +570,7 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
         s = buffers();
     }
     if (s) return s;
+    if (!two_word_slots_fit(c)) exact = false;
     if (!c->table_clean) {
         if ((s = clear_table(c, 0))) return s;
         CK(cudaMemsetAsync(c->bitmap.p, 0, c->bitmap.bytes, c->stream));
@@ -886,33 +891,40 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
 
     bool exact_keys = W <= 2 && n <= 62 && c->opt_exact;
     uint64_t tslots = 0, slot_bytes = 0;
-    // the table of cache_alloc rows, and the candidate rows, which wait in tmp only
-    // when the keys are fingerprints
-    auto ensure_table = [&]() -> rei_status {
-        rei_status s;
-        // (exact keys: the language and its first candidate; else one word)
-        slot_bytes = exact_keys && !use_direct ? 16 : 8;
-        tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
-        const void *before = c->table.p;
-        const size_t before_bytes = c->table.bytes;
-        if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
-        if (c->table.p != before || c->table.bytes != before_bytes) {
-            c->table_clean = false;
-            c->table_extent = c->table.bytes;
-        }
-        return ensure(c, c->tmp, exact_keys ? 4096 : 4ull * W * chunk_max);
-    };
-    // What to do when memory runs out: give back the table (it may be larger than
-    // this search's), and where a slot would be two words go on with one, that is
-    // with fingerprints, in chunks whose rows take half a word a slot at most.  So no
-    // search takes more memory than exact keys would in slots of 12 bytes.
-    auto smaller_table = [&]() -> rei_status {
-        drop_table(c);
-        if (!exact_keys || use_direct) return REI_OK;
+    // fingerprints instead of exact keys: slots of one word, and chunks whose
+    // candidate rows take half a word a slot at most
+    auto fingerprints = [&]() -> rei_status {
         if (use_seen && c->seen.p) CK(cudaMemsetAsync(c->seen.p, 0, c->seen.bytes, c->stream));
         exact_keys = use_seen = false;
         chunk_max = std::min(chunk_max, std::max<uint64_t>(1, table_slots(cache_alloc, cap, chunk_max, n, false) / W));
         return REI_OK;
+    };
+    // the table of cache_alloc rows, and the candidate rows, which wait in tmp only
+    // when the keys are fingerprints
+    auto ensure_table = [&]() -> rei_status {
+        rei_status s;
+        for (;;) {
+            // (exact keys: the language and its first candidate; else one word)
+            slot_bytes = exact_keys && !use_direct ? 16 : 8;
+            tslots = table_slots(cache_alloc, cap, chunk_max, n, use_direct);
+            const void *before = c->table.p;
+            const size_t before_bytes = c->table.bytes;
+            if ((s = ensure(c, c->table, slot_bytes * tslots))) return s;
+            if (c->table.p != before || c->table.bytes != before_bytes) {
+                c->table_clean = false;
+                c->table_extent = c->table.bytes;
+            }
+            if (slot_bytes == 8 || two_word_slots_fit(c)) break;
+            if ((s = fingerprints())) return s;
+        }
+        return ensure(c, c->tmp, exact_keys ? 4096 : 4ull * W * chunk_max);
+    };
+    // What to do when memory runs out: give back the table (it may be larger than
+    // this search's), and where a slot would be two words go on with fingerprints.  So
+    // no search takes more memory than exact keys would in slots of 12 bytes.
+    auto smaller_table = [&]() -> rei_status {
+        drop_table(c);
+        return exact_keys && !use_direct ? fingerprints() : REI_OK;
     };
     // after a fused launch the cache holds its rows: grow keeping them
     auto ensure_rows = [&](DevBuf &b, size_t bytes) {
