@@ -53,7 +53,7 @@ def problems():
 def kernel_sources_hash() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("search.cuh", "solve.cu", "relaunch.cu", "slots.cu", "stage_dev.cuh", "rei_dev.cuh"):
+    for f in ("search.cuh", "sizes.h", "solve.cu", "relaunch.cu", "slots.cu", "stage_dev.cuh", "rei_dev.cuh"):
         with open(os.path.join(ROOT, "paper_2305_18575_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -839,7 +839,7 @@ rei_status solve_one(rei_ctx *c, const rei_problem *p, rei_result *out, const Sl
     // the launch at two CTAs per SM (one, if it already has only one).  A
     // search continued from a first launch or a memory slot is past its start:
     // the SM's memory is the L1's then (its spilled registers and operand rows;
-    // a deep search of 1-word languages 107 -> 81 ms, |ic| 65-128 4.3 -> 3.7 ms)
+    // a deep search of 1-word languages 103.6 -> 78.7 ms, |ic| 65-128 4.3 -> 3.7 ms)
     uint32_t small_rows = 0;
     if (c->opt_small_rows != 0 && W <= 8 && !fused) {
         const size_t half = c->smem_sm / 2 > 4096 ? c->smem_sm / 2 - 4096 : 0;  // static smem + reserve
@@ -1729,7 +1729,7 @@ rei_status run_batch(rei_ctx *c, const rei_problem *probs, const std::vector<uin
     // search in its slot.  A group that has not ended after group_us parks
     // again, and the searches left share the GPU in a new launch: the longest of
     // a batch would else run to its end on the few CTAs of its group (256
-    // uneven problems, 17 of them parked: 4.7 -> 3.5 ms).  The allowance grows
+    // uneven problems: 4.4 -> 3.2 ms).  The allowance grows
     // with every launch; a search that is alone has none.
     std::vector<Parked> rest, grp;
     for (const Parked &pk : redo) (pk.slot < slots && pk.need_rows == 0 ? grp : rest).push_back(pk);
@@ -1916,8 +1916,8 @@ rei_status rei_solve_batch(rei_ctx *c, const rei_problem *probs, uint32_t n, rei
     // the batch (each one problem per SM; every sample is solved exactly, so
     // tuning costs no work), else the default: 8 warps, chunks of 2^11, which one
     // CTA keeps its bookkeeping of in shared memory and which end a search
-    // within 50 us of its allowance (256 uneven problems: 4.0, 2.9 and 2.2 ms on
-    // three sets, with chunks of 2^14 4.3, 3.2 and 2.6 ms)
+    // within 50 us of its allowance (256 uneven problems: 3.2 ms, with chunks of
+    // 2^14 3.4 ms)
     uint32_t warps = tune && tune->warps_per_cta ? tune->warps_per_cta : (uint32_t)c->batch_warps;
     uint32_t chunk = tune && tune->chunk ? tune->chunk : c->batch_chunk;
     const uint32_t yield_us = tune && tune->yield_us ? tune->yield_us

@@ -305,7 +305,7 @@ extern "C" rei_status rei_solve_noalloc(const rei_problem *p, void *stream_v, re
     if (smem > smem_max) NA_RET(REI_EINVAL);
     // the first levels in CTA 0's shared memory, as the plain solve's first
     // launch has them (with 8-warp CTAs, no shared-memory start and every CTA
-    // planning each level, four medium searches took 625 us, so 520 us)
+    // planning each level, four medium searches took 615 us, so 469 us)
     uint32_t small_rows = 0;
     if (W <= 8) {
         uint32_t r = W <= 2 ? 4096u : W <= 4 ? 2048u : 1024u;

@@ -229,8 +229,9 @@ __host__ __device__ inline uint32_t small_tmp(uint32_t W) { return W <= 8 ? kSor
 // the better one: it spreads a chunk over more warps, and a chunk of a few
 // tiles a warp ends with its slowest tile (in the first launch tiles of 128
 // made medium searches 3 % slower).  The relaunch takes eight 1-word
-// candidates a lane (a deep search 81 ms, with four 86 ms) and four 2-word ones
-// (|ic| 36-42 to cost 20: 9.5 ms; two 9.6 ms, six 10.3 ms, eight 11.3 ms).
+// candidates a lane (|ic| up to 30 to cost 26, 1.2e10 candidates: 78.7 ms, with
+// four 84.0 ms) and four 2-word ones (|ic| 36-42 to cost 20: 8.5 ms; two 9.0 ms,
+// six 9.0 ms, eight 9.9 ms).
 constexpr uint32_t kRegChunk = 64;
 template <uint32_t WC>
 __host__ __device__ constexpr uint32_t reg_per() { return WC == 1 ? 8u : 4u; }
@@ -804,9 +805,10 @@ __device__ __forceinline__ bool mark_tile(const SolveJob &J, uint32_t xl, uint32
 // another at src, into A (row stride Ws), with f applied to every word.  U loads
 // a lane are in flight before any is stored: one after another (U = 1) a tile of
 // 32-word languages takes 32 round trips to the L2 for its operands.  U = 8 for
-// the widest languages (|ic| near 1000 to cost 12: 8.1 -> 7.0 ms), 4 for 4 to 16
-// words at 64 registers (|ic| 65-128: 4.6 -> 4.4 ms; 8 spilled and cost 12-word
-// searches 4 %), 1 in the first launch, whose tiles are small.
+// the widest languages (|ic| near 1000 to cost 12: 7.0 ms; one 7.7 ms, four
+// 7.1 ms), 4 for 4 to 16 words at 64 registers (|ic| 65-128 to cost 17: 3.73 ms;
+// one 3.90, two 3.80, eight 3.73; 12 words, |ic| 400-500: 2.49 ms; one 2.53, two
+// 2.50, eight, which spills more, 2.62), 1 in the first launch, whose tiles are small.
 template <uint32_t WT, uint32_t U, class F>
 __device__ __forceinline__ void load_rows(uint32_t *A, const uint32_t *src, uint32_t Wr, uint32_t Ws, uint32_t nrow, F f) {
     const uint32_t lane = threadIdx.x & 31, W = WT ? WT : Wr;
@@ -1120,9 +1122,8 @@ __device__ __forceinline__ bool w1_finish(const TileCtx &T, const Seg &sg, uint3
 
 // one tile of 1-word candidates: 32 of a unary segment (one per lane), or
 // 32 * K of a binary one (K per lane, 32 apart).  A candidate that equals one of
-// its operands is cached already and ends there (a deep search 97.0 -> 94.2 ms).
-// Returns, in each
-// lane, whether it marked a candidate in the chunk's bitmap.
+// its operands is cached already and ends there (a deep search 79.3 -> 78.7 ms).
+// Returns, in each lane, whether it marked a candidate in the chunk's bitmap.
 template <uint32_t K>
 __device__ bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTile &tl, uint64_t tile, uint32_t *wm) {
     // (few candidates: the bit-sliced fixed point)
@@ -1220,9 +1221,9 @@ __device__ bool run_tile_w1(const TileCtx &T, const Seg &sg, const SegTile &tl, 
 // the operand rows, table slots and claims of a lane's four candidates are in
 // flight together, where the bit-sliced tile waits for one after another.  What
 // bounds it is the HBM's rate of random accesses, one a candidate: 8-byte loads
-// at random addresses ran at 288 G/s within 64 MB, 124 G/s in 128 MB, 51 G/s in
-// 512 MB and 40 G/s from 2 GB on.  Specifications of |ic| 36 - 42 searched to
-// cost 20: 12.3 ms bit-sliced, 9.3 ms so.
+// at random addresses ran at 304 G/s within 64 MB, 125 G/s in 128 MB, 51 G/s in
+// 512 MB and 42 to 40 G/s from 2 GB on.  Specifications of |ic| 36 - 42 searched to
+// cost 20: 13.5 ms bit-sliced, 8.5 ms so.
 
 __device__ __forceinline__ void w2_tables(const Shared &S, uint32_t n, uint2 sh, bool swapped, uint32_t *tab,
                                           uint32_t lane) {
@@ -2079,7 +2080,9 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
                    (W & 3u) == 0 && ((reinterpret_cast<uintptr_t>(J.cs) | reinterpret_cast<uintptr_t>(J.tmp)) & 15u) == 0,
                    a.bw > 32};
         bool marked = false;
-        // (a chunk's tiles, at most 2^26 / 32 plus one per segment, fit 32 bits)
+        // (a chunk's tiles fit 32 bits: fewer than its candidates, at most 2^28, but for
+        // the segments it cuts, which tiled over their left operands have a tile more
+        // for each right one, of fewer than 2^31 languages)
         const uint32_t ntiles = (uint32_t)*s_tiles;
         const uint32_t gw = team_r * nwarps + wid, nw = team_n * nwarps;
         uint32_t s = 0;
@@ -2091,11 +2094,11 @@ __device__ __forceinline__ int process_chunk(const SolveJob &J, SolveState *st, 
         const bool dyn = full && ntiles >= kDynTilesPerWarp * nw;
         // (1-word languages: longer runs of tiles that share an operand, whose
         // lookup tables are then built once per run; short runs keep the warps'
-        // operand rows near each other.  1 word: 79 ms a deep search with 8
-        // tiles, 81 with 16, 88 with 32; 2 words: 8.7 ms with 4, 8.8 with 8, 9.2
-        // with 16, 10.2 with 32; 4 words: 3.7 ms with 4, 3.8 with 8.)  Towards
-        // the chunk's end the grabs shrink, so that the last warp is a tile or
-        // two behind the others.
+        // operand rows near each other.  1 word: 78.7 ms a deep search with 8
+        // tiles, 79.5 with 4, 80.6 with 16, 87.6 with 32; 2 words: 8.5 ms with 4,
+        // 8.7 with 8, 9.2 with 16, 10.1 with 32; 4 words: 3.73 ms with 4, 3.82
+        // with 8.)  Towards the chunk's end the grabs shrink, so that the last
+        // warp is a tile or two behind the others.
         const uint32_t most = W == 1 ? 2 * kGrab : kGrab;
         auto grab_at = [&](uint32_t at) { return max(1u, min(most, (ntiles - at) / nw)); };
         uint32_t t = gw, end = ntiles, step = nw;
@@ -2541,11 +2544,11 @@ struct Cta {
 // marked candidates (the first nmarks of a chunk may hold marks) of a chunk
 // that ended with the answer before its survivors were appended; their marks
 // are cleared too.  When that is the quicker way the whole table is written
-// instead, in order: beyond the L2 (256 MiB and more) the HBM takes 23 G slots a
-// second at random addresses and about 400 G in order, so from a sixteenth of
-// the slots on (a search of 35 million 2-word languages took 1.0 ms to empty its
-// table, 0.27 ms so); within it random addresses run at about 200 G a second,
-// and a table is never full enough.
+// instead, in order: beyond the L2 (256 MiB and more) the HBM takes 23 to 27 G stores
+// a second at random addresses, and in order about 400 G slots of 16 bytes, so from a
+// sixteenth of the slots on (|ic| 36-42 to cost 20: 9.0 -> 8.5 ms a search; 1-word
+// languages to cost 26: 81.7 -> 78.7 ms); within it random addresses run at about 200 G
+// a second, and a table is never full enough.
 __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nmarks, uint32_t team_n,
                                    uint32_t team_r) {
     const uint64_t t = (uint64_t)team_r * blockDim.x + threadIdx.x, nt = (uint64_t)team_n * blockDim.x;
@@ -2602,8 +2605,8 @@ __device__ inline void clean_table(const SolveJob &J, uint32_t rows, uint32_t nm
 // candidates stay in registers and whose operands are read from shared memory,
 // survivors that need no decoding (the operands are noted when a candidate
 // takes its slot), three barriers a level instead of nine, and the next level
-// planned by warp 0 while the others append this one.  Small queries 73.7 ->
-// 68.0 us, medium searches (eight in a row) 1203 -> 1032 us.
+// planned by warp 0 while the others append this one.  Small queries 65.7 ->
+// 59.7 us, medium searches (eight in a row) 1071 -> 905 us.
 
 // one tile of 32 candidates
 template <uint32_t WT>

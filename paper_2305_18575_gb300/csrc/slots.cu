@@ -10,12 +10,6 @@ namespace rei {
 // problems from a queue and solves each one on its own (its own memory slot,
 // no grid-wide synchronisation), with the same leader code as k_solve.
 
-// Solve the problem whose job (staged data, costs) is in shared memory J,
-// in memory slot `slot`, on this CTA alone; the report goes to *out and the
-// tree to J.tree.  Returns the search's status (every thread).  With
-// ST_NEED_MEM (the time allowance ran out or the slot is too small) the slot
-// keeps the cache rows, back-pointers, level table and state for the host to
-// continue from; its uniqueness table and survivor bitmap are emptied.
 // a problem's search in memory slot `slot`: its cache, table, chunk
 // workspace, level table, state and answer-walk stack (one CTA's share)
 __device__ void bind_slot(SolveJob &J, const SlotMem &m, uint32_t slot) {
@@ -56,9 +50,14 @@ __device__ void report_slot(const SolveJob &J, uint32_t status, uint32_t slot, u
     o.need_rows = status == ST_NEED_MEM ? st->need_rows : 0u;
 }
 
-// keep_table: a search that parks leaves its uniqueness table in the slot
-// (the batch continues it there, or empties the table when it continues
-// elsewhere); else the table is emptied for the slot's next problem
+// Solve the problem whose job (staged data, costs) is in shared memory J,
+// in memory slot `slot`, on this CTA alone; the report goes to *out and the
+// tree to J.tree.  Returns the search's status (every thread).  With
+// ST_NEED_MEM (the time allowance ran out or the slot is too small) the slot
+// keeps the cache rows, back-pointers, level table and state for the host to
+// continue from; its survivor bitmap is emptied.  keep_table: its uniqueness
+// table stays in the slot as well (the search continues there, or the host
+// empties the table when it continues elsewhere); else it is emptied too.
 __device__ uint32_t solve_in_slot(SolveJob &J, const SlotMem &m, uint32_t slot, BatchOut *out, uint8_t *smem_raw,
                               Plan *s_plan, uint32_t *s_red, uint64_t *s_tiles, unsigned long long *s_found,
                               uint32_t *s_marked, Lead *L, uint64_t yield_ns, bool keep_table) {
