@@ -141,8 +141,8 @@ typedef struct rei_result {
 
 /* Optional device allocator.  alloc returns memory at an 8-byte boundary (at a
  * 16-byte one the uniqueness table can hold exact keys, see above), or NULL on
- * failure.  Both get the context stream; the library frees everything it allocated before
- * rei_ctx_destroy returns. */
+ * failure.  Both get the context stream; the library frees everything it
+ * allocated before rei_ctx_destroy returns. */
 typedef struct rei_alloc {
     void *(*alloc)(void *user, size_t bytes, void *stream);
     void (*free)(void *user, void *ptr, size_t bytes, void *stream);
