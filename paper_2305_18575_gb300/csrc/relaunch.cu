@@ -11,8 +11,8 @@ namespace rei {
 // registers (|ic| 36-42 to cost 20: 8.5 ms, with two CTAs, which spill into the
 // L1, 8.8 ms; 1-word languages, bound by the L2, took 98.1 ms with one instead of
 // 78.7, 4-word ones 4.87 ms instead of 3.73), and from 20 words on, where the warps'
-// tiles leave room for one CTA an SM anyway (32 words to cost 12: 8.3 -> 7.0 ms; 12
-// words 2.49 ms, with one CTA 2.74).
+// tiles leave room for one CTA an SM anyway (32 words to cost 12: 8.3 -> 7.0 ms; 8
+// to 16 words 2.49 ms, with one CTA 2.74).
 // The two CTAs may also be one of 32 warps: searches side by side take one an SM
 // (solve_warps_max).
 template <uint32_t WC>

@@ -807,8 +807,8 @@ __device__ __forceinline__ bool mark_tile(const SolveJob &J, uint32_t xl, uint32
 // 32-word languages takes 32 round trips to the L2 for its operands.  U = 8 for
 // the widest languages (|ic| near 1000 to cost 12: 7.0 ms; one 7.7 ms, four
 // 7.1 ms), 4 for 4 to 16 words at 64 registers (|ic| 65-128 to cost 17: 3.73 ms;
-// one 3.90, two 3.80, eight 3.73; 12 words, |ic| 400-500: 2.49 ms; one 2.53, two
-// 2.50, eight, which spills more, 2.62), 1 in the first launch, whose tiles are small.
+// one 3.90, two 3.80, eight 3.73; 8 to 16 words, |ic| 220-390: 2.49 ms; one 2.53,
+// two 2.50, eight, which spills more, 2.62), 1 in the first launch, whose tiles are small.
 template <uint32_t WT, uint32_t U, class F>
 __device__ __forceinline__ void load_rows(uint32_t *A, const uint32_t *src, uint32_t Wr, uint32_t Ws, uint32_t nrow, F f) {
     const uint32_t lane = threadIdx.x & 31, W = WT ? WT : Wr;

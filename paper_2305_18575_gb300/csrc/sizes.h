@@ -42,7 +42,7 @@ struct Carve {
 // Linear probing of a table of mask + 1 slots from hash h.  No candidate is marked
 // with slot kNoMark, the last of the largest table: the number says that a candidate
 // is not marked, and probing passes the slot over.  (A flag beside the slot instead
-// cost 12-word searches 2 %, medium ones 0.5 %.)
+// cost searches of 8 to 16 words 2 %, medium ones 0.5 %.)
 constexpr uint32_t kNoMark = 0xFFFFFFFFu;
 REI_HD uint32_t probe_first(uint64_t h, uint64_t mask) {
     const uint32_t p = (uint32_t)(h & mask);
