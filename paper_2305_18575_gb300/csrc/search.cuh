@@ -610,7 +610,7 @@ __device__ void dedup_insert_solo(const TileCtx &T, const uint32_t *c, uint32_t 
     const uint64_t h = cs_hash(c, W, 1);
     const uint32_t fp = (uint32_t)(h >> 32);
     const unsigned long long mine = ((uint64_t)fp << 32) | kPending | xl;
-    uint32_t p = probe_first(h, J.table_mask);
+    uint64_t p = probe_first(h, J.table_mask);
     row_write(J.tmp + (uint64_t)xl * W, c, W, T.vec);
     __threadfence_block();
     for (uint64_t probe = 0; probe <= J.table_mask; probe++) {
@@ -633,7 +633,7 @@ __device__ void dedup_insert_solo(const TileCtx &T, const uint32_t *c, uint32_t 
                 return;
             }
         }
-        p = probe_next(p, (uint32_t)J.table_mask);
+        p = probe_next(p, J.table_mask);
     }
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
 }
@@ -741,7 +741,7 @@ __device__ uint32_t dedup_insert(const TileCtx &T, const uint32_t *c, uint32_t x
     const uint64_t h = cs_hash(c, W, 1);
     const uint32_t fp = (uint32_t)(h >> 32);
     const uint64_t mine = ((uint64_t)fp << 32) | kPending | xl;
-    uint32_t p = probe_first(h, J.table_mask);
+    uint64_t p = probe_first(h, J.table_mask);
     bool wrote = false;
     auto write_tmp = [&]() {
         if (wrote) return;
@@ -772,7 +772,7 @@ __device__ uint32_t dedup_insert(const TileCtx &T, const uint32_t *c, uint32_t x
                 return (uint32_t)p;
             }
         }
-        p = probe_next(p, (uint32_t)J.table_mask);
+        p = probe_next(p, J.table_mask);
     }
     atomicExch(&T.st->err, 2u);  // table full: cannot happen with load <= 1/2
     return kNoMark;

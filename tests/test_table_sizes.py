@@ -69,12 +69,14 @@ int main() {
     if (probe_first(0x12345678FFFFFFFFull, top) != top - 1 || probe_first(0x12345678FFFFFFFEull, top) != top - 1) return 1;
     if (probe_next(0xFFFFFFFEu, 0xFFFFFFFFu) != 0 || probe_next(0xFFFFFFFDu, 0xFFFFFFFFu) != 0xFFFFFFFEu) return 2;
     if (probe_next(7u, 0xFFFFFFFFu) != 8) return 3;
+    if (probe_next(top - 1, top) != 0 || probe_next(top - 2, top) != top - 1 || probe_next(uint64_t(7), top) != 8) return 7;
     // any other: every slot in turn
     for (uint64_t bits = 10; bits < 32; bits++) {
         const uint64_t mask = (1ull << bits) - 1;
         const uint32_t m = (uint32_t)mask;
         if (probe_first(~0ull, mask) != mask || probe_first(~0ull - 1, mask) != mask - 1) return 4;
         if (probe_next(m - 1, m) != m || probe_next(m, m) != 0) return 5;
+        if (probe_next(mask - 1, mask) != mask || probe_next(mask, mask) != 0) return 6;
     }
     return 0;
 }
