@@ -508,11 +508,7 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
     const uint64_t chunk_words = c->opt_chunk > 0 ? (uint64_t)c->opt_chunk : (1ull << 22);
     const uint32_t threads = 512;  // (the launch bounds of k_solve_fused: one 16-warp CTA per SM)
     const size_t smem = c->smem_optin > 8192 ? c->smem_optin - 8192 : 0;  // (its static shared memory and a reserve)
-    int bps = 0;
-    CK(solve_fused_occupancy(threads, smem, &bps));
-    if (bps < 1) return REI_EBUSY;
-    uint32_t grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
-    if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
+    uint32_t grid = 0;
     bool exact = c->opt_exact != 0;  // allowed; the launch decides from the staged size
     uint64_t slot_bytes = 16;
     auto buffers = [&]() -> rei_status {
@@ -541,6 +537,11 @@ rei_status run_fused(rei_ctx *c, const rei_problem *p, Staged &sg, double &ms_se
             if ((s = ensure(c, c->bitmap, 4ull * ((chunk_words + 31) / 32)))) return s;
             if (c->bitmap.p != before || c->bitmap.bytes != before_bytes) c->table_clean = false;
         }
+        int bps = 0;
+        CK(solve_fused_occupancy(threads, smem, &bps));
+        if (bps < 1) return REI_EBUSY;
+        grid = std::min<uint32_t>((uint32_t)(std::max(1, c->sm_count / (int)c->share) * bps), kMaxTeam);
+        if (c->opt_grid > 0 && (uint32_t)c->opt_grid < grid) grid = (uint32_t)c->opt_grid;
         if ((s = ensure(c, c->blk, 4ull * grid))) return s;
         if ((s = ensure(c, c->lvl_start, 8ull * (max_cost + 2)))) return s;
         if ((s = ensure(c, c->lvl_count, 8ull * (max_cost + 2)))) return s;
